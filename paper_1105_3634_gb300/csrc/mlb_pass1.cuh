@@ -15,6 +15,7 @@
 #pragma once
 
 #include "mlb_passes.cuh"
+#include "mlb_cube.cuh"
 
 namespace {
 
@@ -301,82 +302,44 @@ __device__ __forceinline__ void pass1_tile_shells(const mlbi_params &p, const ml
     }
 }
 
-// Shell sums for reach 1 by offset class (axis, face, corner): the offsets
-// and unit vectors are compile-time constants and cube_mask selects the
-// classes of each pair's shell.  The +-d data of a class is read once per
-// neighbour species and shared by every species a.  f[3], g[3]: element
-// offsets of the planes z - 1, z, z + 1 of the float4 and dg tiles.
-template <int S, bool DRAG, int CL, bool HC>
-__device__ __forceinline__ void pass1_cube_class(const mlbi_params &p, const float4 *sf, const float *sg, int b,
-                                                 const int (&f)[3], const int (&g)[3], const Centre<S> &c, const float (&ub)[S][3],
-                                                 const PairW<S> &w, Acc1<S> &A)
-{
-    using T = Tile<S, 1>;
-    constexpr float il = cls_il(CL);
-    bool has[S];
-    bool any = false;
-#pragma unroll
-    for (int a = 0; a < S; ++a) {
-        has[a] = (p.cube_mask[pair_of(a, b, S)] >> cls_bit(CL)) & 1;
-        any |= has[a];
-    }
-    if (!any) return;
-    const float nr = p.nref[b];
-    static_for<0, cls_n(CL)>([&](auto I) {
-        constexpr int k = cls_k(CL, decltype(I)::value);
-        constexpr int off = cube_kx(k) + T::TXH * cube_ky(k), dz = cube_kz(k);
-        const float4 vp = sf[f[1 + dz] + b * T::PLANE + off];
-        const float4 vm = sf[f[1 - dz] + b * T::PLANE - off];
-        // the arithmetic of pass1_point with the +d and -d lanes packed
-        const float2 npm = add2(f2(nr, nr), f2(vp.x, vm.x));            // (n(r+d), n(r-d))
-        const float dd = vp.x - vm.x;
-        float2 jpm = f2(0.f, 0.f);                                          // s.u^b(r +- d)
-        if constexpr (!DRAG) {
-            if constexpr (cube_kx(k) != 0) jpm = fma2(f2(cube_kx(k) * il, cube_kx(k) * il), f2(vp.y, vm.y), jpm);
-            if constexpr (cube_ky(k) != 0) jpm = fma2(f2(cube_ky(k) * il, cube_ky(k) * il), f2(vp.z, vm.z), jpm);
-            if constexpr (cube_kz(k) != 0) jpm = fma2(f2(cube_kz(k) * il, cube_kz(k) * il), f2(vp.w, vm.w), jpm);
-        }
-#pragma unroll
-        for (int a = 0; a < S; ++a) {
-            if (!has[a]) continue;
-            const int q = pair_of(a, b, S);
-            const float2 dg2 = f2(sg[g[1 + dz] + q * T::PLANE + off], sg[g[1 - dz] + q * T::PLANE - off]);
-            const float k1 = 0.5f * p.pair[q].vx_pre;
-            const float2 gpm = fma2(f2(k1, k1), dg2, f2(w.kp[q], w.kp[q]));   // exchange weights at r +- d
-            const float2 hpm = mul2(gpm, npm);
-            const float wn = hpm.x + hpm.y;
-            float sd;
-            if constexpr (DRAG) {
-                const float sdu = cube_dot<k>(il, c.u[a][0] - ub[b][0], c.u[a][1] - ub[b][1], c.u[a][2] - ub[b][2]);
-                sd = -wn * sdu;
-            } else {
-                const float su = cube_dot<k>(il, c.u[a][0], c.u[a][1], c.u[a][2]);
-                const float2 j2 = add2(jpm, f2(-su, -su));                   // s.(u^b(r +- d) - u^a(r))
-                sd = fmaf(hpm.x, j2.x, hpm.y * j2.y);
-            }
-            const float t = HC ? fmaf(w.h[q], dd, (-0.5f * p.pair[q].hc_pre) * fmaf(npm.x, dg2.x, -npm.y * dg2.y))
-                               : 0.f;
-            cube_add2<k>(il, f2(t, sd), A.hf[a]);
-            cube_add_ss<k>(il, wn, A.G[a]);
-        }
-    });
-}
-
-template <int S, bool DRAG, bool HC>
+// Shell sums for reach 1 (mlb_cube.cuh), folded into the site's force sums.
+// The exchange sums are relative to the partners' own velocity at r (ub):
+// Gamma_ab (u^b(r) - u^a(r)) completes them.
+template <int S, bool DRAG, int MODE>
 __device__ __forceinline__ void pass1_cube(const mlbi_params &p, const float4 *sf, const float *sg, int kz, int cidx,
-                                           const Centre<S> &c, const float (&ub)[S][3], const PairW<S> &w,
-                                           Acc1<S> &A)
+                                           const Centre<S> &c, const float (&ub)[S][3],
+                                           const float (&dgc)[S * (S + 1) / 2], Acc1<S> &A)
 {
+    constexpr bool HC = MODE == kExact;
     using T = Tile<S, 1>;
-    const int f[3] = {ring(kz - 1, T::NSLOT) * S * T::PLANE + cidx, ring(kz, T::NSLOT) * S * T::PLANE + cidx,
-                      ring(kz + 1, T::NSLOT) * S * T::PLANE + cidx};
-    const int g[3] = {ring(kz - 1, T::NSLOT) * T::NP * T::PLANE + cidx, ring(kz, T::NSLOT) * T::NP * T::PLANE + cidx,
-                      ring(kz + 1, T::NSLOT) * T::NP * T::PLANE + cidx};
+    const CubeView<S> view(sf, sg, kz, cidx, T::NSLOT);
 #pragma unroll
     for (int b = 0; b < S; ++b) {
-        pass1_cube_class<S, DRAG, 0, HC>(p, sf, sg, b, f, g, c, ub, w, A);
-        pass1_cube_class<S, DRAG, 1, HC>(p, sf, sg, b, f, g, c, ub, w, A);
-        pass1_cube_class<S, DRAG, 2, HC>(p, sf, sg, b, f, g, c, ub, w, A);
+        PairSums<S> s;
+        p1_cube_species<S, DRAG, HC>(p, view, b, dgc, ub[b], s);
+#pragma unroll
+        for (int a = 0; a < S; ++a) {
+            const mlbi_pair &pr = p.pair[pair_of(a, b, S)];
+            const float K = 0.5f * pr.vx_pre, H = -0.5f * pr.hc_pre;
+            float E[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) E[k] = K * va_get<S>(s.E[k], a);
+            A.G[a][0] = add2(A.G[a][0], f2(E[0], E[1]));
+            A.G[a][1] = add2(A.G[a][1], f2(E[2], E[3]));
+            A.G[a][2] = add2(A.G[a][2], f2(E[4], E[5]));
+            if constexpr (HC)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) A.hf[a][k].x = fmaf(H, va_get<S>(s.D[k], a), A.hf[a][k].x);
+            if constexpr (!DRAG)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) A.hf[a][k].y = fmaf(K, va_get<S>(s.P[k], a), A.hf[a][k].y);
+            if (MODE == kSweep || a != b) {
+                const float w[3] = {ub[b][0] - c.u[a][0], ub[b][1] - c.u[a][1], ub[b][2] - c.u[a][2]};
+                A.hf[a][0].y = fmaf(E[0], w[0], fmaf(E[3], w[1], fmaf(E[4], w[2], A.hf[a][0].y)));
+                A.hf[a][1].y = fmaf(E[3], w[0], fmaf(E[1], w[1], fmaf(E[5], w[2], A.hf[a][1].y)));
+                A.hf[a][2].y = fmaf(E[4], w[0], fmaf(E[5], w[1], fmaf(E[2], w[2], A.hf[a][2].y)));
+            }
+        }
     }
 }
 
@@ -428,12 +391,15 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
         float dgc[T::NP];
 #pragma unroll
         for (int q = 0; q < T::NP; ++q) dgc[q] = sg[cs * T::NP * T::PLANE + q * T::PLANE + cidx];
-        PairW<S> w;
-        pair_weights<S>(p, dgc, w);
         Acc1<S> A;
         A.zero();
-        if constexpr (R == 1 && TY == kBY) pass1_cube<S, DRAG, HC>(p, sf, sg, kz, cidx, c, ub, w, A);
-        else pass1_tile_shells<S, R, DRAG, TY, HC>(p, stab, sf, sg, kz, cidx, c, ub, w, A);
+        if constexpr (R == 1 && TY == kBY) {
+            pass1_cube<S, DRAG, MODE>(p, sf, sg, kz, cidx, c, ub, dgc, A);
+        } else {
+            PairW<S> w;
+            pair_weights<S>(p, dgc, w);
+            pass1_tile_shells<S, R, DRAG, TY, HC>(p, stab, sf, sg, kz, cidx, c, ub, w, A);
+        }
         if constexpr (MODE == kSweep) {
             sweep_finish<S>(p, r, c, A, frest, pst);
             continue;
@@ -456,8 +422,12 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
     }
 }
 
+// Resident blocks asked for: 4 leaves 128 registers a thread, enough for the
+// cube sums without spills (256^3 binary, reach 1: 0.867 ms; 5 blocks 0.892, 6
+// blocks 0.996, both spilling).  The loads from shared memory bound the kernel
+// (76 % of the L1's wavefronts at 128^3, issue slots 66 %).
 template <int S, int R, bool DRAG, int TY, int MODE>
-__global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes, S <= 2 ? (MODE == kSweep ? 4 : 6) : 2))
+__global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes, S <= 2 ? 4 : 2))
     k_pass1_tiled(const mlbi_params p, const float4 *__restrict__ mom, const float *__restrict__ dg,
                   const mlbi_entry *__restrict__ tab, const float4 *__restrict__ fext, const float4 *__restrict__ attr,
                   const float4 *__restrict__ mom_c, float4 *__restrict__ frest, float4 *__restrict__ pst)
@@ -468,7 +438,7 @@ __global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes, S
 
 // every member of a group (block table entries {member, bx, by, bz}), the exact pass
 template <int S, int R, bool DRAG, int TY>
-__global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes + sizeof(mlbi_params), S <= 2 ? 6 : 2))
+__global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes + sizeof(mlbi_params), S <= 2 ? 4 : 2))
     k_pass1_group(const mlbi_member *__restrict__ mem, const int4 *__restrict__ blk)
 {
     __shared__ mlbi_params sp;

@@ -7,6 +7,7 @@
 // the same thread collides and streams its site right away (the collision
 // needs only the site's own acceleration).
 #include "mlb_passes.cuh"
+#include "mlb_cube.cuh"
 #include "mlb_collide.cuh"
 
 namespace {
@@ -169,72 +170,25 @@ __device__ __forceinline__ void pass2_tile_shells(const mlbi_params &p, const ml
     }
 }
 
-// reach 1 by offset class (see pass1_cube_class)
-template <int S, bool DRAG, int CL>
-__device__ __forceinline__ void pass2_cube_class(const mlbi_params &p, const float4 *sf, const float *sg, int b,
-                                                 const int (&f)[3], const int (&g)[3], const PairW<S> &w,
-                                                 const float (&us)[S][3], float (&acc)[S][3])
-{
-    using T = Tile<S, 1>;
-    constexpr float il = cls_il(CL);
-    bool has[S];
-    bool any = false;
-#pragma unroll
-    for (int a = 0; a < S; ++a) {
-        has[a] = (p.cube_mask[pair_of(a, b, S)] >> cls_bit(CL)) & 1;
-        any |= has[a];
-    }
-    if (!any) return;
-    const float nr = p.nref[b];
-    static_for<0, cls_n(CL)>([&](auto I) {
-        constexpr int k = cls_k(CL, decltype(I)::value);
-        constexpr int off = cube_kx(k) + T::TXH * cube_ky(k), dz = cube_kz(k);
-        const float4 vp = sf[f[1 + dz] + b * T::PLANE + off];
-        const float4 vm = sf[f[1 - dz] + b * T::PLANE - off];
-        // the arithmetic of pass2_point with the +d and -d lanes packed
-        const float2 npm = add2(f2(nr, nr), f2(vp.x, vm.x));
-        float2 jpm = f2(0.f, 0.f);
-        if constexpr (!DRAG) {
-            if constexpr (cube_kx(k) != 0) jpm = fma2(f2(cube_kx(k) * il, cube_kx(k) * il), f2(vp.y, vm.y), jpm);
-            if constexpr (cube_ky(k) != 0) jpm = fma2(f2(cube_ky(k) * il, cube_ky(k) * il), f2(vp.z, vm.z), jpm);
-            if constexpr (cube_kz(k) != 0) jpm = fma2(f2(cube_kz(k) * il, cube_kz(k) * il), f2(vp.w, vm.w), jpm);
-        }
-#pragma unroll
-        for (int a = 0; a < S; ++a) {
-            if (!has[a]) continue;
-            const int q = pair_of(a, b, S);
-            const float2 dg2 = f2(sg[g[1 + dz] + q * T::PLANE + off], sg[g[1 - dz] + q * T::PLANE - off]);
-            const float k1 = 0.5f * p.pair[q].vx_pre;
-            const float2 hpm = mul2(fma2(f2(k1, k1), dg2, f2(w.kp[q], w.kp[q])), npm);
-            float sd;
-            if constexpr (DRAG) {
-                const float sdu = cube_dot<k>(il, us[a][0] - us[b][0], us[a][1] - us[b][1], us[a][2] - us[b][2]);
-                sd = -(hpm.x + hpm.y) * sdu;
-            } else {
-                const float su = cube_dot<k>(il, us[a][0], us[a][1], us[a][2]);
-                const float2 j2 = add2(jpm, f2(-su, -su));
-                sd = fmaf(hpm.x, j2.x, hpm.y * j2.y);
-            }
-            cube_add<k>(il, sd, acc[a]);
-        }
-    });
-}
-
+// reach 1 (mlb_cube.cuh)
 template <int S, bool DRAG, int NSL = 4>
 __device__ __forceinline__ void pass2_cube(const mlbi_params &p, const float4 *sf, const float *sg, int kz, int cidx,
-                                           const PairW<S> &w, const float (&us)[S][3], float (&acc)[S][3])
+                                           const float (&dgc)[S * (S + 1) / 2], const float (&us)[S][3],
+                                           float (&acc)[S][3])
 {
-    using T = Tile<S, 1>;
-    const int f[3] = {ring(kz - 1, NSL) * S * T::PLANE + cidx, ring(kz, NSL) * S * T::PLANE + cidx,
-                      ring(kz + 1, NSL) * S * T::PLANE + cidx};
-    const int g[3] = {ring(kz - 1, NSL) * T::NP * T::PLANE + cidx, ring(kz, NSL) * T::NP * T::PLANE + cidx,
-                      ring(kz + 1, NSL) * T::NP * T::PLANE + cidx};
+    const CubeView<S> view(sf, sg, kz, cidx, NSL);
+    VA<S> ua[3], P[3];
 #pragma unroll
-    for (int b = 0; b < S; ++b) {
-        pass2_cube_class<S, DRAG, 0>(p, sf, sg, b, f, g, w, us, acc);
-        pass2_cube_class<S, DRAG, 1>(p, sf, sg, b, f, g, w, us, acc);
-        pass2_cube_class<S, DRAG, 2>(p, sf, sg, b, f, g, w, us, acc);
+    for (int k = 0; k < 3; ++k) {
+        ua[k] = va_make<S>([&](int a) { return us[a][k]; });
+        P[k] = va_zero<S>();
     }
+#pragma unroll
+    for (int b = 0; b < S; ++b) p2_cube_species<S, DRAG>(p, view, b, dgc, ua, us[b], P);
+#pragma unroll
+    for (int a = 0; a < S; ++a)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) acc[a][k] += va_get<S>(P[k], a);
 }
 
 // the shell sums of the acceleration of the site at ring position kz of the
@@ -248,16 +202,19 @@ __device__ __forceinline__ void pass2_site(const mlbi_params &p, const mlbi_entr
     float dgc[T::NP];
 #pragma unroll
     for (int q = 0; q < T::NP; ++q) dgc[q] = sg[cs * T::NP * T::PLANE + q * T::PLANE + cidx];
-    PairW<S> w;
-    pair_weights<S>(p, dgc, w);
     float us[S][3];
 #pragma unroll
     for (int a = 0; a < S; ++a) {
         const float4 v = sf[cs * S * T::PLANE + a * T::PLANE + cidx];
         us[a][0] = v.y; us[a][1] = v.z; us[a][2] = v.w;
     }
-    if constexpr (R == 1 && TY == kBY) pass2_cube<S, DRAG, NSL>(p, sf, sg, kz, cidx, w, us, acc);
-    else pass2_tile_shells<S, R, DRAG, TY, NSL>(p, tab, sf, sg, kz, cidx, w, us, acc);
+    if constexpr (R == 1 && TY == kBY) {
+        pass2_cube<S, DRAG, NSL>(p, sf, sg, kz, cidx, dgc, us, acc);
+    } else {
+        PairW<S> w;
+        pair_weights<S>(p, dgc, w);
+        pass2_tile_shells<S, R, DRAG, TY, NSL>(p, tab, sf, sg, kz, cidx, w, us, acc);
+    }
 }
 
 template <int S, int R, bool DRAG, int TY>

@@ -242,76 +242,11 @@ __device__ __forceinline__ void stage_plane(const mlbi_params &p, const int (&xy
 // The 13 canonical half offsets (first non-zero of (dz, dy, dx) positive).
 // With reach 1 every contact shell is a union of the three classes |d|^2 = 1
 // (axis), 2 (face diagonal), 3 (corner); the bit of class CL in cube_mask is
-// the bit of its first offset.  All compile-time: the class loops unroll and
-// the unit vectors become immediates.
-__host__ __device__ constexpr int cube_kx(int k) { return k == 0 || k == 3 || k == 6 || k == 9 || k == 12 ? 1 : (k == 1 || k == 4 || k == 7 || k == 10 ? -1 : 0); }
-__host__ __device__ constexpr int cube_ky(int k) { return k == 1 || k == 2 || k == 3 || k == 10 || k == 11 || k == 12 ? 1 : (k >= 4 && k <= 6 ? -1 : 0); }
-__host__ __device__ constexpr int cube_kz(int k) { return k >= 4 ? 1 : 0; }
-__host__ __device__ constexpr int cls_n(int cl) { return cl == 0 ? 3 : (cl == 1 ? 6 : 4); }
+// the bit of its first offset.
 __host__ __device__ constexpr int cls_bit(int cl) { return cl == 0 ? 0 : (cl == 1 ? 1 : 4); }
-__host__ __device__ constexpr int cls_k(int cl, int i)
-{
-    return cl == 0 ? (i == 0 ? 0 : (i == 1 ? 2 : 8)) : (cl == 1 ? 2 * i + 1 : (i < 2 ? 4 + 2 * i : 6 + 2 * i));
-}
 __host__ __device__ constexpr float cls_il(int cl)   // 1/|d|
 {
     return cl == 0 ? 1.0f : (cl == 1 ? 0.70710678118654752f : 0.57735026918962576f);
-}
-
-// s . v for cube offset K (zero components drop out)
-template <int K>
-__device__ __forceinline__ float cube_dot(float il, float vx, float vy, float vz)
-{
-    float r = 0.f;
-    if constexpr (cube_kx(K) != 0) r = fmaf(cube_kx(K) * il, vx, r);
-    if constexpr (cube_ky(K) != 0) r = fmaf(cube_ky(K) * il, vy, r);
-    if constexpr (cube_kz(K) != 0) r = fmaf(cube_kz(K) * il, vz, r);
-    return r;
-}
-
-template <int K>
-__device__ __forceinline__ void cube_add(float il, float t, float (&v)[3])
-{
-    if constexpr (cube_kx(K) != 0) v[0] = fmaf(cube_kx(K) * il, t, v[0]);
-    if constexpr (cube_ky(K) != 0) v[1] = fmaf(cube_ky(K) * il, t, v[1]);
-    if constexpr (cube_kz(K) != 0) v[2] = fmaf(cube_kz(K) * il, t, v[2]);
-}
-
-// (F^hc, F^v) += s (t, sd) for cube offset K, one packed FMA per non-zero component
-template <int K>
-__device__ __forceinline__ void cube_add2(float il, float2 tsd, float2 (&hf)[3])
-{
-    if constexpr (cube_kx(K) != 0) hf[0] = fma2(f2(cube_kx(K) * il, cube_kx(K) * il), tsd, hf[0]);
-    if constexpr (cube_ky(K) != 0) hf[1] = fma2(f2(cube_ky(K) * il, cube_ky(K) * il), tsd, hf[1]);
-    if constexpr (cube_kz(K) != 0) hf[2] = fma2(f2(cube_kz(K) * il, cube_kz(K) * il), tsd, hf[2]);
-}
-
-// G += wn s s^T for cube offset K, G packed as (xx, yy), (zz, xy), (xz, yz);
-// a pair with one zero entry is a scalar FMA on the other lane
-template <int K>
-__device__ __forceinline__ void cube_add_ss(float il, float wn, float2 (&G)[3])
-{
-    constexpr int X = cube_kx(K), Y = cube_ky(K), Z = cube_kz(K);
-    const float i2 = il * il;
-    if constexpr (X != 0 && Y != 0) G[0] = fma2(f2(wn, wn), f2(i2, i2), G[0]);
-    else if constexpr (X != 0) G[0].x = fmaf(wn, i2, G[0].x);
-    else if constexpr (Y != 0) G[0].y = fmaf(wn, i2, G[0].y);
-    if constexpr (Z != 0 && X * Y != 0) G[1] = fma2(f2(wn, wn), f2(i2, X * Y * i2), G[1]);
-    else if constexpr (Z != 0) G[1].x = fmaf(wn, i2, G[1].x);
-    else if constexpr (X * Y != 0) G[1].y = fmaf(wn, X * Y * i2, G[1].y);
-    if constexpr (X * Z != 0 && Y * Z != 0) G[2] = fma2(f2(wn, wn), f2(X * Z * i2, Y * Z * i2), G[2]);
-    else if constexpr (X * Z != 0) G[2].x = fmaf(wn, X * Z * i2, G[2].x);
-    else if constexpr (Y * Z != 0) G[2].y = fmaf(wn, Y * Z * i2, G[2].y);
-}
-
-// compile-time loop: f(std::integral_constant<int, I>) for I = 0 .. N-1
-template <int I, int N, class F>
-__device__ __forceinline__ void static_for(F &&f)
-{
-    if constexpr (I < N) {
-        f(std::integral_constant<int, I>{});
-        static_for<I + 1, N>(f);
-    }
 }
 
 }  // namespace

@@ -1,0 +1,70 @@
+"""The contact-shell sums of both force passes against the FP64 oracle, on the
+lattices where their kernels differ: species counts, offset classes, drag-only
+mode, walls, sizes around the tile edges.
+
+Bounds, as in the parity tests: accelerations of one FP32 force evaluation
+within 1e-4 of the field's largest value, densities and velocities after a few
+steps within 1e-5.
+"""
+import numpy as np
+import pytest
+
+from paper_1105_3634_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+TOL_STATE = 1e-5
+TOL_ACC = 1e-4
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1105_3634_gb300 import build
+    build.build()
+    from paper_1105_3634_gb300 import mlb
+    return mlb
+
+
+def site(a, b):
+    return float(np.abs(a - b).max() / np.abs(b).max())
+
+
+def check(gpu, orc, lat, n, u, steps):
+    sim = gpu.Simulation(lat)
+    sim.set_fields(n, u)
+    f = orc.init(lat, n, u)
+    on, oj = orc.moments(lat, f)
+    assert site(sim.acceleration(), orc.accel(lat, on, oj)) < TOL_ACC
+    sim.step(steps)
+    orc.step(lat, f, steps)
+    gn, gu = sim.moments()
+    on, oj = orc.moments(lat, f)
+    assert site(gn, on) < TOL_STATE
+    assert site(gu, orc.velocity_fields(lat, on, oj)) < TOL_STATE
+    sim.close()
+
+
+def fields(lat, packing, seed=5):
+    n0 = W.densities_from_packing(packing, lat.sigma, [1.0 / lat.nspecies] * lat.nspecies)
+    return W.noise(lat, n0, 0.05, seed), W.random_velocities(lat, 0.02, seed + 1)
+
+
+# reach 1: shells that are unions of axis, face and corner offsets
+CUBE = {
+    "one_axis_face": dict(sigma=[1.0], shape=(33, 5, 14)),
+    "one_all_drag": dict(sigma=[1.5], shape=(31, 9, 3), drag_only=True),
+    "two_mixed_masks": dict(sigma=[1.0, 1.5], shape=(34, 7, 13), wall_axis=2),
+    "three": dict(sigma=[1.0, 1.25, 1.5], shape=(35, 6, 5), wall_axis=0),
+    "three_drag": dict(sigma=[1.0, 1.25, 1.5], shape=(8, 6, 5), drag_only=True),
+    "four": dict(sigma=[1.0, 1.2, 1.4, 1.5], shape=(36, 5, 4)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CUBE))
+def test_cube_shells(gpu, orc, name):
+    lat = W.Lattice(**CUBE[name])
+    n, u = fields(lat, 0.12)
+    check(gpu, orc, lat, n, u, 3)
