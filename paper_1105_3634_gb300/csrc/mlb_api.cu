@@ -134,23 +134,23 @@ EncodeTiledFn encode_tiled()
 }
 
 // TMA descriptors of the populations, moments and rest force for the fused
-// pass-2 + collision kernel: boxes of one 32 x 4 tile row block of one z
+// pass-2 + collision kernel: boxes of one tile (32 x 4 or 16 x 8) of one z
 // plane, all species (and all 19 populations) at once.  Rows of FP32
 // populations must be 16-byte multiples, so nx % 4 == 0; otherwise (or if the
 // driver lacks the call) maps.ok stays 0 and the kernel stages by cp.async.
-void encode_maps(mlb_ctx *c)
+void encode_maps(const mlb_ctx *c, int tile_x, mlbi_maps &m)
 {
-    mlbi_maps &m = c->maps;
     m.ok = 0;
     const mlbi_params &p = c->p;
     EncodeTiledFn fn = encode_tiled();
     if (!fn || p.nx % 4 != 0) return;
     const cuuint64_t nx = p.nx, ny = p.ny, nz = p.nz, S = p.S;
+    const cuuint32_t tx = tile_x, ty = 128 / tile_x;
     const cuuint32_t ones[5] = {1, 1, 1, 1, 1};
     {
         const cuuint64_t dims[4] = {nx, ny, nz, S * MLBI_Q};
         const cuuint64_t strides[3] = {nx * 4, nx * ny * 4, nx * ny * nz * 4};
-        const cuuint32_t box[4] = {32, 4, 1, (cuuint32_t)(S * MLBI_Q)};
+        const cuuint32_t box[4] = {tx, ty, 1, (cuuint32_t)(S * MLBI_Q)};
         for (int k = 0; k < 2; ++k)
             if (fn(&m.f[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, c->b.f[k], dims, strides, box, ones,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -160,7 +160,7 @@ void encode_maps(mlb_ctx *c)
     {
         const cuuint64_t dims[5] = {4, nx, ny, nz, S};
         const cuuint64_t strides[4] = {16, nx * 16, nx * ny * 16, nx * ny * nz * 16};
-        const cuuint32_t box[5] = {4, 32, 4, 1, (cuuint32_t)S};
+        const cuuint32_t box[5] = {4, tx, ty, 1, (cuuint32_t)S};
         if (fn(&m.mom, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, c->b.mom, dims, strides, box, ones,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -499,9 +499,10 @@ mlb_status rebuild(mlb_ctx *c)
         if (p.ball_count[g] != 1) p.local_g = 0;
     p.tile_r = tile_r;
     p.attr_r = attraction ? attr_r : 0;
-    // planes per block of the stencil kernels unless tuned: 12 leaves shorter
-    // last waves than 16 on large lattices (256^3: 0.5 % faster per step)
-    p.zchunk = std::min(c->desc.nz, c->tuned_zchunk > 0 ? c->tuned_zchunk : 12);
+    p.tile_x = mlbi_tile_x(S, tile_r, c->desc.nx, c->desc.ny);
+    p.zchunk = c->tuned_zchunk > 0 ? std::min(c->desc.nz, c->tuned_zchunk)
+                                   : mlbi_planes_per_block(p, mlbi_tile_planes(p));
+    encode_maps(c, p.tile_x, c->maps);
     // the 13 canonical half offsets of the 3x3x3 cube, in the order the kernels use:
     // (1,0,0); (-1,1,0), (0,1,0), (1,1,0); then dz = 1 with dy = -1, 0, 1 and dx = -1, 0, 1
     {
@@ -848,7 +849,6 @@ mlb_status mlb_create(const mlb_lattice_desc *d, mlb_ctx **out)
     c->b.flags = (unsigned int *)q;
     c->b.first_bad = (unsigned long long *)(q + 64);      // in the flags block (256 bytes)
     c->b.maps = &c->maps;
-    encode_maps(c);
     cudaError_t e = cudaMemsetAsync(c->b.flags, 0, sizeof(unsigned int), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->b.fext, 0, sz_v4, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -1439,13 +1439,33 @@ mlb_status build_groups(mlb_batch *b)
     std::vector<std::vector<int4>> tables[3];
     size_t bytes = 0;
     auto take = [&](size_t n) { bytes = (bytes + 255) & ~size_t(255); const size_t o = bytes; bytes += n; return o; };
+    // tile width and planes per block for the lane's whole work (a member alone
+    // would take fewer planes)
+    std::vector<std::vector<mlbi_params>> par;
     for (const auto &g : b->group_members) {
+        std::vector<mlbi_params> q;
+        for (int i : g) q.push_back(b->m[i]->p);
+        long long planes[2] = {0, 0};              // 32 x 4, 16 x 8
+        for (mlbi_params &v : q)
+            for (int k = 0; k < 2; ++k) {
+                v.tile_x = k ? 16 : 32;
+                planes[k] += mlbi_tile_planes(v);
+            }
+        const int w = mlbi_narrow_tiles(q[0].S, q[0].tile_r, planes[0], planes[1]);
+        for (size_t k = 0; k < q.size(); ++k) {
+            q[k].tile_x = w ? 16 : 32;
+            if (b->m[g[k]]->tuned_zchunk <= 0) q[k].zchunk = mlbi_planes_per_block(q[k], planes[w]);
+        }
+        par.push_back(std::move(q));
+    }
+    for (size_t gi = 0; gi < b->group_members.size(); ++gi) {
+        const auto &g = b->group_members[gi];
         off_mem.push_back(take(g.size() * sizeof(mlbi_member)));
         for (int k = 0; k < 3; ++k) {
             std::vector<int4> t;
             for (size_t j = 0; j < g.size(); ++j) {
                 int grid[3];
-                mlbi_group_grid(b->m[g[j]]->p, k, grid);
+                mlbi_group_grid(par[gi][j], k, grid);
                 const long long nb = (long long)grid[0] * grid[1] * grid[2];
                 if (nb + (long long)t.size() > (1ll << 30)) return batch_fail(b, MLB_EINVAL, "group too large");
                 for (long long q = 0; q < nb; ++q) {
@@ -1472,11 +1492,14 @@ mlb_status build_groups(mlb_batch *b)
         for (size_t j = 0; j < g.size(); ++j) {
             const mlb_ctx *c = b->m[g[j]];
             std::memset(static_cast<void *>(&mem[j]), 0, sizeof(mlbi_member));
-            mem[j].map_f[0] = c->maps.f[0];
-            mem[j].map_f[1] = c->maps.f[1];
-            mem[j].map_mom = c->maps.mom;
-            mem[j].map_frest = c->maps.frest;
-            mem[j].p = c->p;
+            mlbi_maps maps;
+            encode_maps(c, par[gi][j].tile_x, maps);
+            if (!maps.ok) return batch_fail(b, MLB_ECUDA, "group tables: tensor maps");
+            mem[j].map_f[0] = maps.f[0];
+            mem[j].map_f[1] = maps.f[1];
+            mem[j].map_mom = maps.mom;
+            mem[j].map_frest = maps.frest;
+            mem[j].p = par[gi][j];
             mem[j].b = c->b;
             mem[j].b.maps = nullptr;
             mem[j].cur = c->cur;
@@ -1494,6 +1517,7 @@ mlb_status build_groups(mlb_batch *b)
         grp.S = q.S;
         grp.R = q.tile_r;
         grp.drag = q.drag_only;
+        grp.tile_x = par[gi][0].tile_x;
         b->groups.push_back(grp);
     }
     if (e != cudaSuccess) return batch_fail(b, MLB_ECUDA, "group tables: %s", cudaGetErrorString(e));

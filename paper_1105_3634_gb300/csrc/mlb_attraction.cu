@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(kBX * TY, 2) k_attraction_columns(const mlbi_p
 {
     using T = CTile<S, R, TY, Z>;
     constexpr int AG = T::AG, W = T::TZH;
+    step_begin();
     extern __shared__ float slab[];                         // [TZH][TYH][TXH]
     const int x0 = blockIdx.x * kBX, y0 = blockIdx.y * TY, z0 = blockIdx.z * Z;
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
@@ -165,8 +166,7 @@ cudaError_t launch_columns(const mlbi_params &p, const mlbi_buffers &b, cudaStre
                  (unsigned)((p.nz + kAttrZ - 1) / kAttrZ));
     const float4 *cols = reinterpret_cast<const float4 *>(b.table) + p.acol_start;
     const float2 *wts = reinterpret_cast<const float2 *>(reinterpret_cast<const float4 *>(b.table) + p.aw_start);
-    k<<<g, dim3(kBX, kAttrTY), T::bytes, s>>>(p, b.mom, cols, wts, b.attr);
-    return cudaGetLastError();
+    return launch_step(k, g, dim3(kBX, kAttrTY), T::bytes, s, p, b.mom, cols, wts, b.attr);
 }
 
 // reach tiers: the smallest tier >= the attraction reach (a wider halo than

@@ -150,9 +150,8 @@ __device__ __forceinline__ VA<S> edot_va(const VA<S> (&u)[3])
 // ------------------------------------------------------------------ the site's view of the staged planes
 // f[k], g[k]: element offsets of plane z - 1 + k at the site, for the float4
 // field of species 0 and the contact-value deviations of pair 0
-template <int S>
+template <int S, class T>
 struct CubeView {
-    using T = Tile<S, 1>;
     const float4 *sf;
     const float *sg;
     int f[3], g[3];
@@ -217,8 +216,8 @@ template <int S, bool DRAG, bool HC>
 struct P1Point {
     VA<S> d, e, p;       // q+ - q-, W+ + W-, W+ j+ + W- j-
     float x;             // n+ - n-
-    template <int X, int Y, int Z>
-    __device__ __forceinline__ void at(const CubeView<S> &c, int b, float nr, const VA<S> &Gc, const float (&ub)[3])
+    template <int X, int Y, int Z, class V>
+    __device__ __forceinline__ void at(const V &c, int b, float nr, const VA<S> &Gc, const float (&ub)[3])
     {
         const float4 vp = c.template field<X, Y, Z>(b), vm = c.template field<-X, -Y, -Z>(b);
         const VA<S> gp = c.template dg<X, Y, Z>(b), gm = c.template dg<-X, -Y, -Z>(b);
@@ -246,8 +245,8 @@ __device__ __forceinline__ void fold_d(const VA<S> &k, const VA<S> &Gc, float x,
     if constexpr (HC) D = va_fma(k, va_fma(x, Gc, d), D);
 }
 
-template <int S, bool DRAG, bool HC>
-__device__ __forceinline__ void p1_axis(const mlbi_params &p, const CubeView<S> &c, int b, float nr, const VA<S> &Gc,
+template <int S, bool DRAG, bool HC, class V>
+__device__ __forceinline__ void p1_axis(const mlbi_params &p, const V &c, int b, float nr, const VA<S> &Gc,
                                         const float (&ub)[3], PairSums<S> &A)
 {
     VA<S> m;
@@ -268,8 +267,8 @@ __device__ __forceinline__ void p1_axis(const mlbi_params &p, const CubeView<S> 
 }
 
 // one plane of face diagonals: components i, j of the vectors, entry ij of the matrix
-template <int S, bool DRAG, bool HC, int I, int J>
-__device__ __forceinline__ void p1_face(const CubeView<S> &c, int b, float nr, const VA<S> &Gc, const float (&ub)[3],
+template <int S, bool DRAG, bool HC, int I, int J, class V>
+__device__ __forceinline__ void p1_face(const V &c, int b, float nr, const VA<S> &Gc, const float (&ub)[3],
                                         const VA<S> &k1, const VA<S> &k2, PairSums<S> &A)
 {
     constexpr int IJ = I + J + 2;                       // xy 3, xz 4, yz 5
@@ -290,8 +289,8 @@ __device__ __forceinline__ void p1_face(const CubeView<S> &c, int b, float nr, c
     }
 }
 
-template <int S, bool DRAG, bool HC>
-__device__ __forceinline__ void p1_corner(const mlbi_params &p, const CubeView<S> &c, int b, float nr, const VA<S> &Gc,
+template <int S, bool DRAG, bool HC, class V>
+__device__ __forceinline__ void p1_corner(const mlbi_params &p, const V &c, int b, float nr, const VA<S> &Gc,
                                           const float (&ub)[3], PairSums<S> &A)
 {
     VA<S> m;
@@ -342,8 +341,8 @@ __device__ __forceinline__ VA<S> twice_g(const mlbi_params &p, const float (&dgc
 }
 
 // sums of neighbour species b
-template <int S, bool DRAG, bool HC>
-__device__ __forceinline__ void p1_cube_species(const mlbi_params &p, const CubeView<S> &c, int b,
+template <int S, bool DRAG, bool HC, class V>
+__device__ __forceinline__ void p1_cube_species(const mlbi_params &p, const V &c, int b,
                                                 const float (&dgc)[S * (S + 1) / 2], const float (&ub)[3],
                                                 PairSums<S> &A)
 {
@@ -366,8 +365,8 @@ __device__ __forceinline__ void p1_cube_species(const mlbi_params &p, const Cube
 // exchange only, at the staged velocities relative to u^a(r) (the friction
 // matrix is not needed, so the relative velocity is taken per a):
 // P = W+ j+ + W- j-, j+- = e.(u^b(r +- d) - u^a(r)); drag only: (W+ + W-) e.(u^b - u^a)(r)
-template <int S, bool DRAG, int X, int Y, int Z>
-__device__ __forceinline__ VA<S> p2_point(const CubeView<S> &c, int b, float nr, const VA<S> &Gc,
+template <int S, bool DRAG, int X, int Y, int Z, class V>
+__device__ __forceinline__ VA<S> p2_point(const V &c, int b, float nr, const VA<S> &Gc,
                                           const VA<S> (&ua)[3], const float (&ub)[3])
 {
     const float4 vp = c.template field<X, Y, Z>(b), vm = c.template field<-X, -Y, -Z>(b);
@@ -386,8 +385,8 @@ __device__ __forceinline__ VA<S> p2_point(const CubeView<S> &c, int b, float nr,
 }
 
 // adds to P[3] the exchange sums of neighbour species b
-template <int S, bool DRAG>
-__device__ __forceinline__ void p2_cube_species(const mlbi_params &p, const CubeView<S> &c, int b,
+template <int S, bool DRAG, class V>
+__device__ __forceinline__ void p2_cube_species(const mlbi_params &p, const V &c, int b,
                                                 const float (&dgc)[S * (S + 1) / 2], const VA<S> (&ua)[3],
                                                 const float (&ub)[3], VA<S> (&P)[3])
 {

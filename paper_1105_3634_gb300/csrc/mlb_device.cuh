@@ -170,6 +170,48 @@ __device__ __forceinline__ int wrap_or_out(int c, int L, bool wall)
 // ring slot of plane z0 - R + k
 __device__ __forceinline__ int ring(int k, int nslot) { return k % nslot; }
 
+// ------------------------------------------------------------------ dependent launches
+// On lattices of up to 2^20 sites the kernels of a time step are launched with
+// programmatic stream serialization: the next kernel's blocks come up while the
+// last ones of the kernel before it still run, and wait in step_begin() for
+// that kernel to complete (and its writes to be visible) before they touch
+// memory.  Every thread of every block calls it first, so a kernel never
+// completes before the one ahead of it.  Measured per step: 64 x 8 x 8 19.8 ->
+// 13.0 us, 97 x 61 x 45 91.3 -> 86.0, 96^3 179 -> 175; 128^3 367 -> 369 and
+// 256^3 2651 -> 2734 (blocks that wait take the place of blocks that run),
+// hence the limit.
+__device__ __forceinline__ void step_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// Plain stream order beyond that and while the stream is captured.
+constexpr long long kDependentSites = 1ll << 20;
+template <class... P, class... A>
+inline cudaError_t launch_step(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                               const mlbi_params &p, A &&...args)
+{
+    bool dependent = p.N <= kDependentSites;
+    if (dependent) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(s, &cap);
+        if (e != cudaSuccess) return e;
+        dependent = cap == cudaStreamCaptureStatusNone;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, p, static_cast<A &&>(args)...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ centre moments
 template <int S>
 struct Centre {

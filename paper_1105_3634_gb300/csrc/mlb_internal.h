@@ -69,6 +69,7 @@ struct mlbi_params {
     // E the largest |dz| any pair reaches on the column; their weights are float2
     // (k, dz k) per (column, pair, dz = 0..attr_r) at ((float2 *)(table + aw_start))
     int acol_start, acol_count, aw_start;
+    int tile_x;                      // tile width of the reach-1 passes of one and two species: 32 (x 4) or 16 (x 8)
     int zchunk;                      // planes per block of the tiled kernels
     int hc_from_attr;                // 1: pass 1 skips the hard-core sums and takes attr as F^hc (surrogate)
     int pair_index[MLBI_MAXS][MLBI_MAXS];
@@ -102,6 +103,47 @@ __host__ __device__ constexpr int mlbi_tile_ty(int S, int R)
          : R < 3 ? (mlbi_tile_bytes(S, R, 4) <= MLBI_MAX_TILE_BYTES && mlbi_tile_warps(S, R, 4) >= 8 ? 4 : 0)
          : mlbi_tile_bytes(S, R, 8) <= MLBI_MAX_TILE_BYTES ? 8
          : (mlbi_tile_bytes(S, R, 4) <= MLBI_MAX_TILE_BYTES && mlbi_tile_warps(S, R, 4) >= 8 ? 4 : 0);
+}
+
+// ------------------------------------------------------------------ work decomposition of the tiled passes
+// Tile width of the reach-1 passes (one and two species): 32 x 4 sites, or 16
+// x 8 where that leaves at least a tenth fewer idle threads (nx = 16: half of a
+// 32-wide tile is idle; nx = 97, ny = 61: 72 % against 83 % of the threads have
+// a site).  At equal use 32 x 4 is the faster: the contact values of a warp's
+// two 16-site rows share banks.
+inline bool mlbi_narrow_tiles(int S, int tile_r, long long tiles32, long long tiles16)
+{
+    return S <= 2 && tile_r == 1 && 10 * tiles16 <= 9 * tiles32;
+}
+inline int mlbi_tile_x(int S, int tile_r, int nx, int ny)
+{
+    return mlbi_narrow_tiles(S, tile_r, (long long)((nx + 31) / 32) * ((ny + 3) / 4),
+                             (long long)((nx + 15) / 16) * ((ny + 7) / 8))
+               ? 16
+               : 32;
+}
+// rows of a tile of pass 1 and of the fused pass 2 + collision
+inline int mlbi_tile_rows(const mlbi_params &p) { return p.tile_r == 1 ? 128 / p.tile_x : mlbi_tile_ty(p.S, p.tile_r); }
+// tile planes (one tile of one z plane) of a lattice
+inline long long mlbi_tile_planes(const mlbi_params &p)
+{
+    const int ty = mlbi_tile_rows(p);
+    return ty < 1 ? 0 : (long long)((p.nx + p.tile_x - 1) / p.tile_x) * ((p.ny + ty - 1) / ty) * p.nz;
+}
+// Planes per block.  A block pays about one plane's time for filling its ring,
+// and the kernel's last blocks run about one block's time with the GPU
+// emptying: with W tile planes on M resident blocks the time goes as
+// W (1 + 1/z)/M + z + 1, least at z = sqrt(W / M).  Measured (reach 1, planes
+// per block and ms per step): 64 x 8 x 8 1: 0.020, 8: 0.056; 97 x 61 x 45 2:
+// 0.094, 12: 0.177; 128^3 6: 0.387, 12: 0.397; 256 x 16^3 4: 0.436, 12: 0.521.
+constexpr int kMlbiSMs = 152;
+inline int mlbi_planes_per_block(const mlbi_params &p, long long tile_planes)
+{
+    const int resident = p.tile_r == 1 ? 4 : (p.tile_r == 2 ? 2 : 1);
+    int z = 1;
+    while (z < 16 && (long long)(2 * z + 1) * (2 * z + 1) * kMlbiSMs * resident < 4 * tile_planes) ++z;   // nearest to the root
+    const int chunks = p.nz > z ? (2 * p.nz + z) / (2 * z) : 1;
+    return (p.nz + chunks - 1) / chunks;
 }
 
 // Bulk tensor (TMA) descriptors of the buffers the fused pass-2 + collision
@@ -224,7 +266,7 @@ struct mlbi_group {
     const mlbi_member *mem;          // [nmem] device
     const int4 *blk[3];              // per stage: [nblk] {member, block x, block y, block z} device
     int nblk[3];                     // (moments: {member, block, blocks of the member, 0})
-    int S, R, drag;                  // the shared instantiation: species, shell reach (1, 2), drag only
+    int S, R, drag, tile_x;          // the shared instantiation: species, shell reach (1, 2), drag only, tile width
 };
 enum { MLBI_GROUP_MOMENTS = 0, MLBI_GROUP_PASS1 = 1, MLBI_GROUP_PASS2 = 2 };
 // whether a member can join a group, and its stage grids (blocks per stage)

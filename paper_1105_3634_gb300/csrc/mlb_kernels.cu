@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(kBlock) k_moments(const mlbi_params p, const f
                                                     float4 *__restrict__ mom, double *__restrict__ partial,
                                                     unsigned int *__restrict__ flags)
 {
+    step_begin();
     const long long N = p.N;
     ConsSums<S> cs;
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < N;
@@ -113,6 +114,7 @@ __global__ void __launch_bounds__(kBX * kBY) k_gfield(mlbi_params p, const float
                                                       const mlbi_entry *__restrict__ tab, float *__restrict__ dg,
                                                       unsigned int *__restrict__ flags)
 {
+    step_begin();
     Loc L;
     if (!locate(p, L)) return;
     const long long N = p.N, r = L.r;
@@ -166,6 +168,7 @@ __global__ void __launch_bounds__(kBlock) k_moments_g(const mlbi_params p, const
                                                       float4 *__restrict__ mom, float *__restrict__ dg,
                                                       unsigned int *__restrict__ flags, double *__restrict__ partial)
 {
+    step_begin();
     moments_g_blocks<S, SUMS>(p, f, mom, dg, flags, partial, blockIdx.x, gridDim.x);
 }
 
@@ -187,6 +190,7 @@ __global__ void __launch_bounds__(kBX * kBY, 6) k_collide(const mlbi_params p, c
                                                           float *__restrict__ fout, const float4 *__restrict__ mom,
                                                           const float4 *__restrict__ accf)
 {
+    step_begin();
     Loc L;
     if (!locate(p, L)) return;
     const long long N = p.N, r = L.r;
@@ -325,15 +329,15 @@ cudaError_t mlbi_launch_moments(const mlbi_params &p, const mlbi_buffers &b, int
         k_conservation_final<<<1, kFinalThreads, 0, s>>>(p, b.partial, MLBI_RED_BLOCKS, b.sums);
         return cudaGetLastError();
     }
-    MLBI_DISPATCH_S((k_moments<SS, false><<<grid_for(p.N), kBlock, 0, s>>>(p, b.f[cur], b.mom, nullptr, nullptr)));
-    return cudaGetLastError();
+    MLBI_DISPATCH_S(return (launch_step(k_moments<SS, false>, grid_for(p.N), kBlock, 0, s, p, b.f[cur], b.mom, nullptr,
+                                        nullptr)));
+    return cudaErrorInvalidValue;
 }
 
 
 cudaError_t mlbi_launch_gfield(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s)
 {
-    k_gfield<<<tiled_grid(p), dim3(kBX, kBY), 0, s>>>(p, b.mom, b.table, b.dg, b.flags);
-    return cudaGetLastError();
+    return launch_step(k_gfield, tiled_grid(p), dim3(kBX, kBY), 0, s, p, b.mom, b.table, b.dg, b.flags);
 }
 
 namespace {
@@ -367,9 +371,9 @@ cudaError_t mlbi_launch_moments_g(const mlbi_params &p, const mlbi_buffers &b, i
         k_conservation_final<<<1, kFinalThreads, 0, s>>>(p, b.partial, MLBI_RED_BLOCKS, b.sums);
         return cudaGetLastError();
     }
-    MLBI_DISPATCH_S((k_moments_g<SS, false><<<grid_for(p.N), kBlock, 0, s>>>(p, b.f[cur], b.mom, b.dg, b.flags,
-                                                                             nullptr)));
-    return cudaGetLastError();
+    MLBI_DISPATCH_S(return (launch_step(k_moments_g<SS, false>, grid_for(p.N), kBlock, 0, s, p, b.f[cur], b.mom, b.dg,
+                                        b.flags, nullptr)));
+    return cudaErrorInvalidValue;
 }
 
 struct V3 {
@@ -473,8 +477,8 @@ cudaError_t mlbi_launch_field_check(const mlbi_params &p, const mlbi_buffers &b,
 cudaError_t mlbi_launch_collide(const mlbi_params &p, const mlbi_buffers &b, int cur, cudaStream_t s)
 {
     const dim3 g = tiled_grid(p), t(kBX, kBY);
-    MLBI_DISPATCH_S((k_collide<SS><<<g, t, 0, s>>>(p, b.f[cur], b.f[cur ^ 1], b.mom, b.acc)));
-    return cudaGetLastError();
+    MLBI_DISPATCH_S(return (launch_step(k_collide<SS>, g, t, 0, s, p, b.f[cur], b.f[cur ^ 1], b.mom, b.acc)));
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t mlbi_launch_init(const mlbi_params &p, const mlbi_buffers &b, int cur, const double *n,

@@ -7,20 +7,7 @@ namespace {
 template <int S, int R, bool DRAG, int MODE = kExact>
 cudaError_t launch_pass1_tiled(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s)
 {
-    constexpr int TY = mlbi_tile_ty(S, R);
-    if constexpr (TY == 0) {
-        return cudaErrorInvalidValue;
-    } else {
-        using T = Tile<S, R, TY>;
-        auto k = k_pass1_tiled<S, R, DRAG, TY, MODE>;
-        const size_t bytes = T::bytes + staged_table_bytes<T, R>(p);
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        const dim3 g((unsigned)((p.nx + kBX - 1) / kBX), (unsigned)((p.ny + TY - 1) / TY),
-                     (unsigned)((p.nz + p.zchunk - 1) / p.zchunk));
-        k<<<g, dim3(kBX, TY), bytes, s>>>(p, b.mom, b.dg, b.table, b.fext, b.attr, b.mom, b.frest, b.pst);
-        return cudaGetLastError();
-    }
+    return launch_tiled<S, R, DRAG, MODE>(p, b, b.mom, b.pst, s);
 }
 
 template <int S, bool DRAG>
@@ -37,23 +24,24 @@ cudaError_t launch_pass1(const mlbi_params &p, const mlbi_buffers &b, cudaStream
     if (p.tile_r == 1) return launch_pass1_tiled<S, 1, DRAG>(p, b, s);
     if (p.tile_r == 2) return launch_pass1_tiled<S, 2, DRAG>(p, b, s);
     if (p.tile_r == 3) return launch_pass1_tiled<S, 3, DRAG>(p, b, s);
-    k_pass1<S, DRAG, kExact><<<tiled_grid(p), dim3(kBX, kBY), 0, s>>>(p, b.mom, b.dg, b.table, b.fext, b.attr, b.mom,
-                                                                        b.frest, b.pst);
-    return cudaGetLastError();
+    return launch_step(k_pass1<S, DRAG, kExact>, tiled_grid(p), dim3(kBX, kBY), 0, s, p, b.mom, b.dg, b.table, b.fext,
+                       b.attr, b.mom, b.frest, b.pst);
 }
 
-template <int S, int R, bool DRAG>
+template <int S, int R, bool DRAG, int TX = kBX>
 cudaError_t launch_pass1_group(const mlbi_group &g, cudaStream_t s)
 {
-    constexpr int TY = mlbi_tile_ty(S, R);
+    constexpr int TY = TX == kBX ? mlbi_tile_ty(S, R) : 128 / TX;
     if constexpr (TY == 0) {
         return cudaErrorInvalidValue;
     } else {
-        using T = Tile<S, R, TY>;
-        auto k = k_pass1_group<S, R, DRAG, TY>;
+        if constexpr (TX == kBX && R == 1)
+            if (g.tile_x == 16) return launch_pass1_group<S, R, DRAG, 16>(g, s);
+        using T = Tile<S, R, TY, TX>;
+        auto k = k_pass1_group<S, R, DRAG, TY, TX>;
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::bytes);
         if (e != cudaSuccess) return e;
-        k<<<(unsigned)g.nblk[MLBI_GROUP_PASS1], dim3(kBX, TY), T::bytes, s>>>(g.mem, g.blk[MLBI_GROUP_PASS1]);
+        k<<<(unsigned)g.nblk[MLBI_GROUP_PASS1], dim3(kBX, T::NT / kBX), T::bytes, s>>>(g.mem, g.blk[MLBI_GROUP_PASS1]);
         return cudaGetLastError();
     }
 }

@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(kBX * kBY) k_pass1(const mlbi_params p, const 
                                                      float4 *__restrict__ pst)
 {
     constexpr int NP = S * (S + 1) / 2;
+    step_begin();
     Loc L;
     if (!locate(p, L)) return;
     const long long N = p.N, r = L.r;
@@ -305,14 +306,13 @@ __device__ __forceinline__ void pass1_tile_shells(const mlbi_params &p, const ml
 // Shell sums for reach 1 (mlb_cube.cuh), folded into the site's force sums.
 // The exchange sums are relative to the partners' own velocity at r (ub):
 // Gamma_ab (u^b(r) - u^a(r)) completes them.
-template <int S, bool DRAG, int MODE>
+template <int S, bool DRAG, int MODE, class T>
 __device__ __forceinline__ void pass1_cube(const mlbi_params &p, const float4 *sf, const float *sg, int kz, int cidx,
                                            const Centre<S> &c, const float (&ub)[S][3],
                                            const float (&dgc)[S * (S + 1) / 2], Acc1<S> &A)
 {
     constexpr bool HC = MODE == kExact;
-    using T = Tile<S, 1>;
-    const CubeView<S> view(sf, sg, kz, cidx, T::NSLOT);
+    const CubeView<S, T> view(sf, sg, kz, cidx, T::NSLOT);
 #pragma unroll
     for (int b = 0; b < S; ++b) {
         PairSums<S> s;
@@ -347,7 +347,7 @@ __device__ __forceinline__ void pass1_cube(const mlbi_params &p, const float4 *s
 // is the previous sweep's (n - n_ref, u*) field, mom_c the moments, frest is
 // read, pst receives the sweep's u*)
 // the tile (bx, by, bz) of the tiled pass 1
-template <int S, int R, bool DRAG, int TY, int MODE>
+template <int S, int R, bool DRAG, int TY, int TX, int MODE>
 __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *__restrict__ mom,
                                            const float *__restrict__ dg, const mlbi_entry *__restrict__ tab,
                                            const float4 *__restrict__ fext, const float4 *__restrict__ attr,
@@ -355,28 +355,28 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
                                            float4 *__restrict__ pst, int bx, int by, int bz)
 {
     constexpr bool HC = MODE == kExact;
-    using T = Tile<S, R, TY>;
+    using T = Tile<S, R, TY, TX>;
     extern __shared__ float4 smem[];
     float4 *sf = smem;                                                      // [NSLOT][S][PLANE]
     float *sg = reinterpret_cast<float *>(smem + (size_t)T::NSLOT * S * T::PLANE);   // [NSLOT][NP][PLANE]
-    const int x0 = bx * kBX, y0 = by * TY, z0 = bz * p.zchunk;
+    const int x0 = bx * TX, y0 = by * TY, z0 = bz * p.zchunk;
     const int z1 = min(z0 + p.zchunk, p.nz);
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+    const int x = x0 + T::lx(), y = y0 + T::ly();
     const bool active = x < p.nx && y < p.ny;
-    const int cidx = (threadIdx.y + R) * T::TXH + threadIdx.x + R;
+    const int cidx = (T::ly() + R) * T::TXH + T::lx() + R;
     const mlbi_entry *stab =
         stage_table<T, R>(p, tab, reinterpret_cast<float4 *>(reinterpret_cast<char *>(smem) + T::bytes));
     int xy[T::J];
-    stage_sites<S, R, TY>(p, x0, y0, xy);
+    stage_sites<T, R>(p, x0, y0, xy);
     for (int k = 0; k < 2 * R + 1; ++k)
-        stage_plane<S, R, TY>(p, xy, z0 - R + k, ring(k, T::NSLOT), mom, dg, sf, sg);
+        stage_plane<T, S>(p, xy, z0 - R + k, ring(k, T::NSLOT), mom, dg, sf, sg);
     cp_async_commit();
     for (int z = z0; z < z1; ++z) {
         cp_async_wait_all();
         __syncthreads();
         const int kz = z - z0 + R;                      // ring position of plane z
         if (z + 1 < z1) {
-            stage_plane<S, R, TY>(p, xy, z + R + 1, ring(kz + R + 1, T::NSLOT), mom, dg, sf, sg);
+            stage_plane<T, S>(p, xy, z + R + 1, ring(kz + R + 1, T::NSLOT), mom, dg, sf, sg);
             cp_async_commit();
         }
         if (!active) continue;
@@ -393,8 +393,8 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
         for (int q = 0; q < T::NP; ++q) dgc[q] = sg[cs * T::NP * T::PLANE + q * T::PLANE + cidx];
         Acc1<S> A;
         A.zero();
-        if constexpr (R == 1 && TY == kBY) {
-            pass1_cube<S, DRAG, MODE>(p, sf, sg, kz, cidx, c, ub, dgc, A);
+        if constexpr (R == 1) {
+            pass1_cube<S, DRAG, MODE, T>(p, sf, sg, kz, cidx, c, ub, dgc, A);
         } else {
             PairW<S> w;
             pair_weights<S>(p, dgc, w);
@@ -426,19 +426,20 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
 // cube sums without spills (256^3 binary, reach 1: 0.867 ms; 5 blocks 0.892, 6
 // blocks 0.996, both spilling).  The loads from shared memory bound the kernel
 // (76 % of the L1's wavefronts at 128^3, issue slots 66 %).
-template <int S, int R, bool DRAG, int TY, int MODE>
-__global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes, S <= 2 ? 4 : 2))
+template <int S, int R, bool DRAG, int TY, int TX, int MODE>
+__global__ void __launch_bounds__(TX * TY, tile_blocks(Tile<S, R, TY, TX>::bytes, S <= 2 ? 4 : 2))
     k_pass1_tiled(const mlbi_params p, const float4 *__restrict__ mom, const float *__restrict__ dg,
                   const mlbi_entry *__restrict__ tab, const float4 *__restrict__ fext, const float4 *__restrict__ attr,
                   const float4 *__restrict__ mom_c, float4 *__restrict__ frest, float4 *__restrict__ pst)
 {
-    pass1_tile<S, R, DRAG, TY, MODE>(p, mom, dg, tab, fext, attr, mom_c, frest, pst, blockIdx.x, blockIdx.y,
+    step_begin();
+    pass1_tile<S, R, DRAG, TY, TX, MODE>(p, mom, dg, tab, fext, attr, mom_c, frest, pst, blockIdx.x, blockIdx.y,
                                      blockIdx.z);
 }
 
 // every member of a group (block table entries {member, bx, by, bz}), the exact pass
-template <int S, int R, bool DRAG, int TY>
-__global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes + sizeof(mlbi_params), S <= 2 ? 4 : 2))
+template <int S, int R, bool DRAG, int TY, int TX>
+__global__ void __launch_bounds__(TX * TY, tile_blocks(Tile<S, R, TY, TX>::bytes + sizeof(mlbi_params), S <= 2 ? 4 : 2))
     k_pass1_group(const mlbi_member *__restrict__ mem, const int4 *__restrict__ blk)
 {
     __shared__ mlbi_params sp;
@@ -446,8 +447,30 @@ __global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes + 
     const mlbi_member *m = mem + e.x;
     group_params(m, sp);
     const mlbi_buffers &b = m->b;
-    pass1_tile<S, R, DRAG, TY, kExact>(sp, b.mom, b.dg, b.table, b.fext, b.attr, b.mom, b.frest, b.pst, e.y, e.z,
+    pass1_tile<S, R, DRAG, TY, TX, kExact>(sp, b.mom, b.dg, b.table, b.fext, b.attr, b.mom, b.frest, b.pst, e.y, e.z,
                                        e.w);
+}
+
+// launch the tiled pass 1 (or sweep: fld the previous sweep's field, out the next) of a lattice
+template <int S, int R, bool DRAG, int MODE, int TX = kBX>
+cudaError_t launch_tiled(const mlbi_params &p, const mlbi_buffers &b, const float4 *fld, float4 *out, cudaStream_t s)
+{
+    constexpr int TY = TX == kBX ? mlbi_tile_ty(S, R) : 128 / TX;
+    if constexpr (TY == 0) {
+        return cudaErrorInvalidValue;
+    } else {
+        if constexpr (TX == kBX && R == 1 && S <= 2)
+            if (p.tile_x == 16) return launch_tiled<S, R, DRAG, MODE, 16>(p, b, fld, out, s);
+        using T = Tile<S, R, TY, TX>;
+        auto k = k_pass1_tiled<S, R, DRAG, TY, TX, MODE>;
+        const size_t bytes = T::bytes + staged_table_bytes<T, R>(p);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+        const dim3 g((unsigned)((p.nx + TX - 1) / TX), (unsigned)((p.ny + TY - 1) / TY),
+                     (unsigned)((p.nz + p.zchunk - 1) / p.zchunk));
+        return launch_step(k, g, dim3(kBX, T::NT / kBX), bytes, s, p, fld, b.dg, b.table, b.fext, b.attr, b.mom, b.frest,
+                           out);
+    }
 }
 
 }  // namespace

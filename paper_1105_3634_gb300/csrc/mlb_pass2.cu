@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(kBX * kBY) k_pass2(const mlbi_params p, const 
                                                      double *__restrict__ acc_out)
 {
     constexpr int NP = S * (S + 1) / 2;
+    step_begin();
     Loc L;
     if (!locate(p, L)) return;
     const long long N = p.N, r = L.r;
@@ -171,12 +172,12 @@ __device__ __forceinline__ void pass2_tile_shells(const mlbi_params &p, const ml
 }
 
 // reach 1 (mlb_cube.cuh)
-template <int S, bool DRAG, int NSL = 4>
+template <int S, bool DRAG, class T, int NSL = 4>
 __device__ __forceinline__ void pass2_cube(const mlbi_params &p, const float4 *sf, const float *sg, int kz, int cidx,
                                            const float (&dgc)[S * (S + 1) / 2], const float (&us)[S][3],
                                            float (&acc)[S][3])
 {
-    const CubeView<S> view(sf, sg, kz, cidx, NSL);
+    const CubeView<S, T> view(sf, sg, kz, cidx, NSL);
     VA<S> ua[3], P[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -193,11 +194,10 @@ __device__ __forceinline__ void pass2_cube(const mlbi_params &p, const float4 *s
 
 // the shell sums of the acceleration of the site at ring position kz of the
 // tile (centre slot cs), added to acc
-template <int S, int R, bool DRAG, int TY, int NSL = 2 * R + 2>
+template <class T, int S, int R, bool DRAG, int NSL = 2 * R + 2>
 __device__ __forceinline__ void pass2_site(const mlbi_params &p, const mlbi_entry *tab, const float4 *sf,
                                            const float *sg, int kz, int cidx, float (&acc)[S][3])
 {
-    using T = Tile<S, R, TY>;
     const int cs = ring(kz, NSL);
     float dgc[T::NP];
 #pragma unroll
@@ -208,50 +208,51 @@ __device__ __forceinline__ void pass2_site(const mlbi_params &p, const mlbi_entr
         const float4 v = sf[cs * S * T::PLANE + a * T::PLANE + cidx];
         us[a][0] = v.y; us[a][1] = v.z; us[a][2] = v.w;
     }
-    if constexpr (R == 1 && TY == kBY) {
-        pass2_cube<S, DRAG, NSL>(p, sf, sg, kz, cidx, dgc, us, acc);
+    if constexpr (R == 1) {
+        pass2_cube<S, DRAG, T, NSL>(p, sf, sg, kz, cidx, dgc, us, acc);
     } else {
         PairW<S> w;
         pair_weights<S>(p, dgc, w);
-        pass2_tile_shells<S, R, DRAG, TY, NSL>(p, tab, sf, sg, kz, cidx, w, us, acc);
+        pass2_tile_shells<S, R, DRAG, T::TY, NSL>(p, tab, sf, sg, kz, cidx, w, us, acc);
     }
 }
 
-template <int S, int R, bool DRAG, int TY>
-__global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes, S <= 2 ? 4 : 2))
+template <int S, int R, bool DRAG, int TY, int TX>
+__global__ void __launch_bounds__(TX * TY, tile_blocks(Tile<S, R, TY, TX>::bytes, S <= 2 ? 4 : 2))
     k_pass2_tiled(const mlbi_params p, const float *__restrict__ dg, const mlbi_entry *__restrict__ tab,
                   const float4 *__restrict__ frest, const float4 *__restrict__ pst, float4 *__restrict__ acc_f,
                   double *__restrict__ acc_out)
 {
-    using T = Tile<S, R, TY>;
+    using T = Tile<S, R, TY, TX>;
+    step_begin();
     extern __shared__ float4 smem[];
     float4 *sf = smem;
     float *sg = reinterpret_cast<float *>(smem + (size_t)T::NSLOT * S * T::PLANE);
-    const int x0 = blockIdx.x * kBX, y0 = blockIdx.y * TY, z0 = blockIdx.z * p.zchunk;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * p.zchunk;
     const int z1 = min(z0 + p.zchunk, p.nz);
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+    const int x = x0 + T::lx(), y = y0 + T::ly();
     const bool active = x < p.nx && y < p.ny;
-    const int cidx = (threadIdx.y + R) * T::TXH + threadIdx.x + R;
+    const int cidx = (T::ly() + R) * T::TXH + T::lx() + R;
     const mlbi_entry *stab =
         stage_table<T, R>(p, tab, reinterpret_cast<float4 *>(reinterpret_cast<char *>(smem) + T::bytes));
     int xy[T::J];
-    stage_sites<S, R, TY>(p, x0, y0, xy);
+    stage_sites<T, R>(p, x0, y0, xy);
     for (int k = 0; k < 2 * R + 1; ++k)
-        stage_plane<S, R, TY>(p, xy, z0 - R + k, ring(k, T::NSLOT), pst, dg, sf, sg);
+        stage_plane<T, S>(p, xy, z0 - R + k, ring(k, T::NSLOT), pst, dg, sf, sg);
     cp_async_commit();
     for (int z = z0; z < z1; ++z) {
         cp_async_wait_all();
         __syncthreads();
         const int kz = z - z0 + R;
         if (z + 1 < z1) {
-            stage_plane<S, R, TY>(p, xy, z + R + 1, ring(kz + R + 1, T::NSLOT), pst, dg, sf, sg);
+            stage_plane<T, S>(p, xy, z + R + 1, ring(kz + R + 1, T::NSLOT), pst, dg, sf, sg);
             cp_async_commit();
         }
         if (!active) continue;
         const long long r = x + (long long)p.nx * (y + (long long)p.ny * z);
         float acc[S][3];
         zero_acc<S>(acc);
-        pass2_site<S, R, DRAG, TY>(p, stab, sf, sg, kz, cidx, acc);
+        pass2_site<T, S, R, DRAG>(p, stab, sf, sg, kz, cidx, acc);
 #pragma unroll
         for (int a = 0; a < S; ++a) add_rest(acc[a], frest[a * p.N + r]);
         store_acc<S>(p, r, acc, acc_f, acc_out);
@@ -268,9 +269,9 @@ __global__ void __launch_bounds__(kBX * TY, tile_blocks(Tile<S, R, TY>::bytes, S
 //   P(z) = the site's populations and moments of plane z.
 // They alternate A(z), P(z), A(z+1), P(z+1), ..., so "all but the newest
 // group" is A(z) at the top of plane z and P(z) before its collision.
-template <int S, int R>
+template <int S, int R, int TX = kBX>
 struct FusedTile {
-    using T = Tile<S, R>;
+    using T = Tile<S, R, 128 / TX, TX>;
     static constexpr size_t pops_off = T::bytes;                                   // float [S*19][NT]
     static constexpr size_t mom_off = pops_off + (size_t)S * MLBI_Q * T::NT * sizeof(float);   // float4 [S][NT]
     static constexpr size_t rest_off = mom_off + (size_t)S * T::NT * sizeof(float4);           // float4 [S][NT]
@@ -301,7 +302,7 @@ __device__ __forceinline__ void stage_rest(const mlbi_params &p, long long r, in
 
 __device__ __forceinline__ void cp_async_wait_all_but_newest() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-template <int S, int R, bool DRAG>
+template <int S, int R, bool DRAG, int TX>
 __global__ void __launch_bounds__(kBX * kBY, S <= 2 ? 3 : 2) k_pass2_collide(const mlbi_params p,
                                                                             const float *__restrict__ dg,
                                                                             const mlbi_entry *__restrict__ tab,
@@ -311,24 +312,25 @@ __global__ void __launch_bounds__(kBX * kBY, S <= 2 ? 3 : 2) k_pass2_collide(con
                                                                             const float *__restrict__ fin,
                                                                             float *__restrict__ fout)
 {
-    using T = Tile<S, R>;
-    using F = FusedTile<S, R>;
+    using F = FusedTile<S, R, TX>;
+    using T = typename F::T;
+    step_begin();
     extern __shared__ float4 smem[];
     float4 *sf = smem;
     float *sg = reinterpret_cast<float *>(smem + (size_t)T::NSLOT * S * T::PLANE);
     float *sF = reinterpret_cast<float *>(reinterpret_cast<char *>(smem) + F::pops_off);
     float4 *sM = reinterpret_cast<float4 *>(reinterpret_cast<char *>(smem) + F::mom_off);
     float4 *sR = reinterpret_cast<float4 *>(reinterpret_cast<char *>(smem) + F::rest_off);
-    const int x0 = blockIdx.x * kBX, y0 = blockIdx.y * kBY, z0 = blockIdx.z * p.zchunk;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * T::TY, z0 = blockIdx.z * p.zchunk;
     const int z1 = min(z0 + p.zchunk, p.nz);
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-    const int tid = threadIdx.y * kBX + threadIdx.x;
+    const int x = x0 + T::lx(), y = y0 + T::ly();
+    const int tid = T::tid();
     const bool active = x < p.nx && y < p.ny;
-    const int cidx = (threadIdx.y + R) * T::TXH + threadIdx.x + R;
+    const int cidx = (T::ly() + R) * T::TXH + T::lx() + R;
     const long long sxy = x + (long long)p.nx * y, nxy = (long long)p.nx * p.ny;
     int xy[T::J];
-    stage_sites<S, R>(p, x0, y0, xy);
-    for (int k = 0; k < 2 * R + 1; ++k) stage_plane<S, R>(p, xy, z0 - R + k, ring(k, T::NSLOT), pst, dg, sf, sg);
+    stage_sites<T, R>(p, x0, y0, xy);
+    for (int k = 0; k < 2 * R + 1; ++k) stage_plane<T, S>(p, xy, z0 - R + k, ring(k, T::NSLOT), pst, dg, sf, sg);
     if (active) stage_rest<S>(p, sxy + nxy * z0, tid, T::NT, frest, sR);
     cp_async_commit();                                                  // A(z0)
     if (active) stage_pops<S>(p, sxy + nxy * z0, tid, T::NT, fin, mom, sF, sM);
@@ -349,12 +351,12 @@ __global__ void __launch_bounds__(kBX * kBY, S <= 2 ? 3 : 2) k_pass2_collide(con
             }
         }
         if (z + 1 < z1) {
-            stage_plane<S, R>(p, xy, z + R + 1, ring(kz + R + 1, T::NSLOT), pst, dg, sf, sg);
+            stage_plane<T, S>(p, xy, z + R + 1, ring(kz + R + 1, T::NSLOT), pst, dg, sf, sg);
             if (active) stage_rest<S>(p, r + nxy, tid, T::NT, frest, sR);
         }
         cp_async_commit();                                              // A(z + 1)
         if (active) {
-            pass2_site<S, R, DRAG, kBY>(p, tab, sf, sg, kz, cidx, acc);
+            pass2_site<T, S, R, DRAG>(p, tab, sf, sg, kz, cidx, acc);
 #pragma unroll
             for (int a = 0; a < S; ++a) add_rest(acc[a], make_float4(rest[a][0], rest[a][1], rest[a][2], 0.f));
         }
@@ -389,9 +391,9 @@ __global__ void __launch_bounds__(kBX * kBY, S <= 2 ? 3 : 2) k_pass2_collide(con
 // sums (a second barrier per plane), and lands during the collisions.  The
 // 9 KB this saves (R = 1, S = 2) and a 128-register bound give 4 resident
 // blocks per SM instead of 3.
-template <int S, int R>
+template <int S, int R, int TX = kBX>
 struct TmaTile {
-    using T = Tile<S, R>;
+    using T = Tile<S, R, 128 / TX, TX>;
     static constexpr int NSL = 2 * R + 1;
     static constexpr size_t pad(size_t b) { return (b + 127) / 128 * 128; }
     static constexpr size_t ring_bytes = (size_t)NSL * T::PLANE * (S * sizeof(float4) + T::NP * sizeof(float));
@@ -406,7 +408,7 @@ struct TmaTile {
 
 // the tile (bx, by, bz) of the fused pass; the maps are kernel parameters or
 // (grouped launches) global-memory copies the issuing thread has acquired
-template <int S, int R, bool DRAG>
+template <int S, int R, bool DRAG, int TX>
 __device__ __forceinline__ void pass2_collide_tma_tile(const mlbi_params &p, const float *__restrict__ dg,
                                                        const mlbi_entry *__restrict__ tab,
                                                        const float4 *__restrict__ pst, float *__restrict__ fout,
@@ -414,8 +416,8 @@ __device__ __forceinline__ void pass2_collide_tma_tile(const mlbi_params &p, con
                                                        const CUtensorMap *map_mom, const CUtensorMap *map_rest,
                                                        int bx, int by, int bz)
 {
-    using T = Tile<S, R>;
-    using F = TmaTile<S, R>;
+    using F = TmaTile<S, R, TX>;
+    using T = typename F::T;
     extern __shared__ float4 smem_raw[];
     __shared__ __align__(8) uint64_t bar_mem;
     // the bulk copies want 128-byte aligned destinations
@@ -428,12 +430,12 @@ __device__ __forceinline__ void pass2_collide_tma_tile(const mlbi_params &p, con
     float4 *sR = reinterpret_cast<float4 *>(base + F::rest_off);
     __shared__ int s_fail;                                       // a wait gave up (read after a barrier)
     const uint32_t bar = smem_u32(&bar_mem);
-    const int x0 = bx * kBX, y0 = by * kBY, z0 = bz * p.zchunk;
+    const int x0 = bx * TX, y0 = by * T::TY, z0 = bz * p.zchunk;
     const int z1 = min(z0 + p.zchunk, p.nz);
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-    const int tid = threadIdx.y * kBX + threadIdx.x;
+    const int x = x0 + T::lx(), y = y0 + T::ly();
+    const int tid = T::tid();
     const bool active = x < p.nx && y < p.ny;
-    const int cidx = (threadIdx.y + R) * T::TXH + threadIdx.x + R;
+    const int cidx = (T::ly() + R) * T::TXH + T::lx() + R;
     const int sxy = x + p.nx * y, nxy = p.nx * p.ny;
     auto issue = [&](int z) {
         mbar_expect_tx(bar, F::tx_bytes);
@@ -446,8 +448,8 @@ __device__ __forceinline__ void pass2_collide_tma_tile(const mlbi_params &p, con
         s_fail = 0;
     }
     int xy[T::J];
-    stage_sites<S, R>(p, x0, y0, xy);
-    for (int k = 0; k < 2 * R + 1; ++k) stage_plane<S, R>(p, xy, z0 - R + k, ring(k, NSL), pst, dg, sf, sg);
+    stage_sites<T, R>(p, x0, y0, xy);
+    for (int k = 0; k < 2 * R + 1; ++k) stage_plane<T, S>(p, xy, z0 - R + k, ring(k, NSL), pst, dg, sf, sg);
     cp_async_commit();
     __syncthreads();                                            // the barrier is initialised
     if (tid == 0) issue(z0);
@@ -460,9 +462,9 @@ __device__ __forceinline__ void pass2_collide_tma_tile(const mlbi_params &p, con
         const int kz = z - z0 + R;
         float acc[S][3];
         zero_acc<S>(acc);
-        if (active) pass2_site<S, R, DRAG, kBY, NSL>(p, tab, sf, sg, kz, cidx, acc);
+        if (active) pass2_site<T, S, R, DRAG, NSL>(p, tab, sf, sg, kz, cidx, acc);
         __syncthreads();              // every thread is done with plane z - R: its slot takes plane z + R + 1
-        if (z + 1 < z1) stage_plane<S, R>(p, xy, z + R + 1, ring(kz + R + 1, NSL), pst, dg, sf, sg);
+        if (z + 1 < z1) stage_plane<T, S>(p, xy, z + R + 1, ring(kz + R + 1, NSL), pst, dg, sf, sg);
         cp_async_commit();
         // each thread waits for the copies itself, so warps move on to their
         // collisions independently; a wait that gives up marks the block failed,
@@ -491,20 +493,21 @@ __device__ __forceinline__ void pass2_collide_tma_tile(const mlbi_params &p, con
     if (s_fail && tid == 0) mbar_wait(bar, phase ^ 1u);       // one more bounded wait for the copy in flight
 }
 
-template <int S, int R, bool DRAG>
+template <int S, int R, bool DRAG, int TX>
 __global__ void __launch_bounds__(kBX * kBY, S <= 2 ? 4 : 2)
     k_pass2_collide_tma(const mlbi_params p, const float *__restrict__ dg, const mlbi_entry *__restrict__ tab,
                         const float4 *__restrict__ pst, float *__restrict__ fout, unsigned int *__restrict__ flags,
                         const __grid_constant__ CUtensorMap map_f, const __grid_constant__ CUtensorMap map_mom,
                         const __grid_constant__ CUtensorMap map_rest)
 {
-    pass2_collide_tma_tile<S, R, DRAG>(p, dg, tab, pst, fout, flags, &map_f, &map_mom, &map_rest, blockIdx.x,
+    step_begin();
+    pass2_collide_tma_tile<S, R, DRAG, TX>(p, dg, tab, pst, fout, flags, &map_f, &map_mom, &map_rest, blockIdx.x,
                                        blockIdx.y, blockIdx.z);
 }
 
 // every member of a group (block table entries {member, bx, by, bz}); odd:
 // the members read f[cur ^ 1] and write f[cur]
-template <int S, int R, bool DRAG>
+template <int S, int R, bool DRAG, int TX>
 __global__ void __launch_bounds__(kBX * kBY, S <= 2 ? 4 : 2)
     k_pass2_collide_group(const mlbi_member *__restrict__ mem, const int4 *__restrict__ blk, int odd)
 {
@@ -519,26 +522,27 @@ __global__ void __launch_bounds__(kBX * kBY, S <= 2 ? 4 : 2)
     }
     group_params(m, sp);
     const mlbi_buffers &b = m->b;
-    pass2_collide_tma_tile<S, R, DRAG>(sp, b.dg, b.table, b.pst, b.f[rd ^ 1], b.flags, &m->map_f[rd], &m->map_mom,
+    pass2_collide_tma_tile<S, R, DRAG, TX>(sp, b.dg, b.table, b.pst, b.f[rd ^ 1], b.flags, &m->map_f[rd], &m->map_mom,
                                        &m->map_frest, e.y, e.z, e.w);
 }
 
-template <int S, int R, bool DRAG>
+template <int S, int R, bool DRAG, int TX = kBX>
 cudaError_t launch_pass2_tiled(const mlbi_params &p, const mlbi_buffers &b, double *acc_out, cudaStream_t s)
 {
-    constexpr int TY = mlbi_tile_ty(S, R);
+    constexpr int TY = TX == kBX ? mlbi_tile_ty(S, R) : 128 / TX;
     if constexpr (TY == 0) {
         return cudaErrorInvalidValue;
     } else {
-        using T = Tile<S, R, TY>;
-        auto k = k_pass2_tiled<S, R, DRAG, TY>;
+        if constexpr (TX == kBX && R == 1 && S <= 2)
+            if (p.tile_x == 16) return launch_pass2_tiled<S, R, DRAG, 16>(p, b, acc_out, s);
+        using T = Tile<S, R, TY, TX>;
+        auto k = k_pass2_tiled<S, R, DRAG, TY, TX>;
         const size_t bytes = T::bytes + staged_table_bytes<T, R>(p);
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e != cudaSuccess) return e;
-        const dim3 g((unsigned)((p.nx + kBX - 1) / kBX), (unsigned)((p.ny + TY - 1) / TY),
+        const dim3 g((unsigned)((p.nx + TX - 1) / TX), (unsigned)((p.ny + TY - 1) / TY),
                      (unsigned)((p.nz + p.zchunk - 1) / p.zchunk));
-        k<<<g, dim3(kBX, TY), bytes, s>>>(p, b.dg, b.table, b.frest, b.pst, b.acc, acc_out);
-        return cudaGetLastError();
+        return launch_step(k, g, dim3(kBX, T::NT / kBX), bytes, s, p, b.dg, b.table, b.frest, b.pst, b.acc, acc_out);
     }
 }
 
@@ -548,39 +552,38 @@ cudaError_t launch_pass2(const mlbi_params &p, const mlbi_buffers &b, double *ac
     if (p.tile_r == 1) return launch_pass2_tiled<S, 1, DRAG>(p, b, acc_out, s);
     if (p.tile_r == 2) return launch_pass2_tiled<S, 2, DRAG>(p, b, acc_out, s);
     if (p.tile_r == 3) return launch_pass2_tiled<S, 3, DRAG>(p, b, acc_out, s);
-    k_pass2<S, DRAG><<<tiled_grid(p), dim3(kBX, kBY), 0, s>>>(p, b.dg, b.table, b.frest, b.pst, b.acc, acc_out);
-    return cudaGetLastError();
+    return launch_step(k_pass2<S, DRAG>, tiled_grid(p), dim3(kBX, kBY), 0, s, p, b.dg, b.table, b.frest, b.pst, b.acc,
+                       acc_out);
 }
 
 constexpr size_t kMaxSharedPerBlock = 227 * 1024;
 
-template <int S, int R, bool DRAG>
+template <int S, int R, bool DRAG, int TX = kBX>
 cudaError_t launch_pass2_collide_tiled(const mlbi_params &p, const mlbi_buffers &b, int cur, cudaStream_t s)
 {
-    using F = FusedTile<S, R>;
+    using F = FusedTile<S, R, TX>;
+    using G = TmaTile<S, R, TX>;
     if constexpr (F::bytes > kMaxSharedPerBlock) {
         return cudaErrorInvalidValue;
     } else {
-    if constexpr (TmaTile<S, R>::bytes <= kMaxSharedPerBlock) {
-        if (b.maps && b.maps->ok) {
-            using G = TmaTile<S, R>;
-            auto k = k_pass2_collide_tma<S, R, DRAG>;
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::bytes);
-            if (e != cudaSuccess) return e;
-            const dim3 g((unsigned)((p.nx + kBX - 1) / kBX), (unsigned)((p.ny + kBY - 1) / kBY),
-                         (unsigned)((p.nz + p.zchunk - 1) / p.zchunk));
-            k<<<g, dim3(kBX, kBY), G::bytes, s>>>(p, b.dg, b.table, b.pst, b.f[cur ^ 1], b.flags, b.maps->f[cur],
-                                                  b.maps->mom, b.maps->frest);
-            return cudaGetLastError();
+        if constexpr (TX == kBX && R == 1 && S <= 2)
+            if (p.tile_x == 16) return launch_pass2_collide_tiled<S, R, DRAG, 16>(p, b, cur, s);
+        const dim3 g((unsigned)((p.nx + TX - 1) / TX), (unsigned)((p.ny + F::T::TY - 1) / F::T::TY),
+                     (unsigned)((p.nz + p.zchunk - 1) / p.zchunk));
+        if constexpr (G::bytes <= kMaxSharedPerBlock) {
+            if (b.maps && b.maps->ok) {
+                auto k = k_pass2_collide_tma<S, R, DRAG, TX>;
+                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::bytes);
+                if (e != cudaSuccess) return e;
+                return launch_step(k, g, dim3(kBX, kBY), G::bytes, s, p, b.dg, b.table, b.pst, b.f[cur ^ 1], b.flags,
+                                   b.maps->f[cur], b.maps->mom, b.maps->frest);
+            }
         }
-    }
-    auto k = k_pass2_collide<S, R, DRAG>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::bytes);
-    if (e != cudaSuccess) return e;
-    const dim3 g((unsigned)((p.nx + kBX - 1) / kBX), (unsigned)((p.ny + kBY - 1) / kBY),
-                 (unsigned)((p.nz + p.zchunk - 1) / p.zchunk));
-    k<<<g, dim3(kBX, kBY), F::bytes, s>>>(p, b.dg, b.table, b.frest, b.pst, b.mom, b.f[cur], b.f[cur ^ 1]);
-    return cudaGetLastError();
+        auto k = k_pass2_collide<S, R, DRAG, TX>;
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::bytes);
+        if (e != cudaSuccess) return e;
+        return launch_step(k, g, dim3(kBX, kBY), F::bytes, s, p, b.dg, b.table, b.frest, b.pst, b.mom, b.f[cur],
+                           b.f[cur ^ 1]);
     }
 }
 
@@ -600,14 +603,16 @@ cudaError_t launch_pass2_collide(const mlbi_params &p, const mlbi_buffers &b, in
     return cudaErrorInvalidValue;          // the global-memory pass 2 is not fused
 }
 
-template <int S, int R, bool DRAG>
+template <int S, int R, bool DRAG, int TX = kBX>
 cudaError_t launch_pass2_collide_group(const mlbi_group &g, int odd, cudaStream_t s)
 {
-    using G = TmaTile<S, R>;
+    using G = TmaTile<S, R, TX>;
     if constexpr (G::bytes + sizeof(mlbi_params) > kMaxSharedPerBlock) {
         return cudaErrorInvalidValue;
     } else {
-        auto k = k_pass2_collide_group<S, R, DRAG>;
+        if constexpr (TX == kBX && R == 1)
+            if (g.tile_x == 16) return launch_pass2_collide_group<S, R, DRAG, 16>(g, odd, s);
+        auto k = k_pass2_collide_group<S, R, DRAG, TX>;
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::bytes);
         if (e != cudaSuccess) return e;
         k<<<(unsigned)g.nblk[MLBI_GROUP_PASS2], dim3(kBX, kBY), G::bytes, s>>>(g.mem, g.blk[MLBI_GROUP_PASS2], odd);
@@ -648,8 +653,8 @@ void mlbi_group_grid(const mlbi_params &p, int stage, int grid[3])
         grid[0] = (int)grid_for(p.N);
         grid[1] = grid[2] = 1;
     } else {
-        const int ty = stage == MLBI_GROUP_PASS1 ? mlbi_tile_ty(p.S, p.tile_r) : kBY;
-        grid[0] = (p.nx + kBX - 1) / kBX;
+        const int ty = mlbi_tile_rows(p);      // reach 1, 2: the same tiles in both passes
+        grid[0] = (p.nx + p.tile_x - 1) / p.tile_x;
         grid[1] = (p.ny + ty - 1) / ty;
         grid[2] = zc;
     }

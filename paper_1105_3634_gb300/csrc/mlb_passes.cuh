@@ -123,16 +123,20 @@ __device__ __forceinline__ Nb fetch_nb(const mlbi_params &p, const Loc &L, const
 // of (32 + 2R) x (TY + 2R) sites: 2R + 1 planes in use and one more being
 // filled by cp.async while the current plane is computed.  Every shell
 // neighbour is then read from shared memory.
-template <int S, int R, int TY_ = kBY>
+template <int S, int R, int TY_ = kBY, int TX_ = kBX>
 struct Tile {
-    static constexpr int TX = kBX, TY = TY_;
+    static constexpr int TX = TX_, TY = TY_;
     static constexpr int TXH = TX + 2 * R, TYH = TY + 2 * R, PLANE = TXH * TYH;
     static constexpr int NSLOT = 2 * R + 2;
     static constexpr int NP = S * (S + 1) / 2;
-    static constexpr int NT = kBX * TY;
+    static constexpr int NT = TX * TY;
     static constexpr int J = (PLANE + NT - 1) / NT;          // staging sites per thread and plane
     static constexpr size_t bytes = (size_t)NSLOT * PLANE * (S * sizeof(float4) + NP * sizeof(float));
-    static_assert(bytes == (size_t)mlbi_tile_bytes(S, R, TY), "tile size formula");
+    static_assert(TX != kBX || bytes == (size_t)mlbi_tile_bytes(S, R, TY), "tile size formula");
+    // this thread's site of the tile
+    static __device__ __forceinline__ int tid() { return threadIdx.y * kBX + threadIdx.x; }
+    static __device__ __forceinline__ int lx() { return TX == kBX ? threadIdx.x : tid() % TX; }
+    static __device__ __forceinline__ int ly() { return TX == kBX ? threadIdx.y : tid() / TX; }
 };
 
 // The shell entries of the table-driven reach-3 tiles, staged once per block
@@ -182,11 +186,10 @@ constexpr int tile_blocks(size_t bytes, int cap)
 
 // (x, y) offsets x + nx y of this thread's staging sites, fixed while the
 // block marches up z; -1 beyond a wall
-template <int S, int R, int TY = kBY>
-__device__ __forceinline__ void stage_sites(const mlbi_params &p, int x0, int y0, int (&xy)[Tile<S, R, TY>::J])
+template <class T, int R>
+__device__ __forceinline__ void stage_sites(const mlbi_params &p, int x0, int y0, int (&xy)[T::J])
 {
-    using T = Tile<S, R, TY>;
-    const int tid = threadIdx.y * kBX + threadIdx.x;
+    const int tid = T::tid();
 #pragma unroll
     for (int j = 0; j < T::J; ++j) {
         const int idx = tid + j * T::NT;
@@ -207,14 +210,13 @@ __device__ __forceinline__ int wrap_plane(int c, int L, bool wall)
 // Stage plane gz of the tile into ring slot `slot`.  Sites beyond a wall get
 // n = 0 (n - n_ref = -n_ref) and zero velocity; their dg is never used (every
 // term carries n(r+d) = 0) and is set to 0.
-template <int S, int R, int TY = kBY>
-__device__ __forceinline__ void stage_plane(const mlbi_params &p, const int (&xy)[Tile<S, R, TY>::J], int gz,
-                                            int slot, const float4 *__restrict__ fld, const float *__restrict__ dg,
-                                            float4 *sf, float *sg)
+template <class T, int S>
+__device__ __forceinline__ void stage_plane(const mlbi_params &p, const int (&xy)[T::J], int gz, int slot,
+                                            const float4 *__restrict__ fld, const float *__restrict__ dg, float4 *sf,
+                                            float *sg)
 {
-    using T = Tile<S, R, TY>;
     const long long N = p.N;
-    const int tid = threadIdx.y * kBX + threadIdx.x;
+    const int tid = T::tid();
     const int z = wrap_plane(gz, p.nz, p.wall_axis == 2);
     const long long zoff = (long long)p.nx * p.ny * z;
 #pragma unroll

@@ -13,20 +13,7 @@ template <int S, int R, bool DRAG>
 cudaError_t launch_sweep_tiled(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next,
                                cudaStream_t s)
 {
-    constexpr int TY = mlbi_tile_ty(S, R);
-    if constexpr (TY == 0) {
-        return cudaErrorInvalidValue;
-    } else {
-        using T = Tile<S, R, TY>;
-        auto k = k_pass1_tiled<S, R, DRAG, TY, kSweep>;
-        const size_t bytes = T::bytes + staged_table_bytes<T, R>(p);
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        const dim3 g((unsigned)((p.nx + kBX - 1) / kBX), (unsigned)((p.ny + TY - 1) / TY),
-                     (unsigned)((p.nz + p.zchunk - 1) / p.zchunk));
-        k<<<g, dim3(kBX, TY), bytes, s>>>(p, prev, b.dg, b.table, b.fext, b.attr, b.mom, b.frest, next);
-        return cudaGetLastError();
-    }
+    return launch_tiled<S, R, DRAG, kSweep>(p, b, prev, next, s);
 }
 
 template <int S, bool DRAG>
@@ -35,9 +22,8 @@ cudaError_t launch_sweep(const mlbi_params &p, const mlbi_buffers &b, const floa
     if (p.tile_r == 1) return launch_sweep_tiled<S, 1, DRAG>(p, b, prev, next, s);
     if (p.tile_r == 2) return launch_sweep_tiled<S, 2, DRAG>(p, b, prev, next, s);
     if (p.tile_r == 3) return launch_sweep_tiled<S, 3, DRAG>(p, b, prev, next, s);
-    k_pass1<S, DRAG, kSweep><<<tiled_grid(p), dim3(kBX, kBY), 0, s>>>(p, prev, b.dg, b.table, b.fext, b.attr, b.mom,
-                                                                        b.frest, next);
-    return cudaGetLastError();
+    return launch_step(k_pass1<S, DRAG, kSweep>, tiled_grid(p), dim3(kBX, kBY), 0, s, p, prev, b.dg, b.table, b.fext,
+                       b.attr, b.mom, b.frest, next);
 }
 
 }  // namespace

@@ -68,3 +68,27 @@ def test_cube_shells(gpu, orc, name):
     lat = W.Lattice(**CUBE[name])
     n, u = fields(lat, 0.12)
     check(gpu, orc, lat, n, u, 3)
+
+
+# tiles of 16 x 8 sites (nx that leaves 32-wide tiles idle), full, one short and one over
+NARROW = {
+    "full": dict(sigma=[1.0, 1.5], shape=(16, 8, 6)),
+    "short": dict(sigma=[1.0, 1.5], shape=(47, 15, 5), wall_axis=1),
+    "over": dict(sigma=[1.5], shape=(12, 9, 19), drag_only=True),
+    "many": dict(sigma=[1.0, 1.5], shape=(80, 40, 33), wall_axis=0),
+}
+
+
+@pytest.mark.parametrize("name", sorted(NARROW))
+def test_narrow_tiles(gpu, orc, name):
+    lat = W.Lattice(**NARROW[name])
+    n, u = fields(lat, 0.12)
+    check(gpu, orc, lat, n, u, 3)
+    out = []
+    for split in (False, True):                       # fused and split launches agree bit for bit
+        sim = gpu.Simulation(lat, split_collide=split)
+        sim.set_fields(n, u)
+        sim.step(4)
+        out.append(sim.populations()[0])
+        sim.close()
+    assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
