@@ -108,8 +108,43 @@ struct SharedPops {
     __device__ __forceinline__ float operator()(int a, int i) const { return f[(a * MLBI_Q + i) * nt]; }
 };
 
-template <int S, class Pops>
-__device__ __forceinline__ void collide_push(const mlbi_params &p, int x, int y, int z, long long r,
+// c.v for a link with components in {-1, 0, 1}, and v.w.  The collision's
+// arithmetic is spelled out (fmaf, __fmul_rn, __fadd_rn) so that no kernel that
+// includes it contracts it differently.
+__device__ __forceinline__ float cdot(int cx, int cy, int cz, float v0, float v1, float v2)
+{
+    float s = 0.f;
+    bool any = false;
+    if (cx) s = cx > 0 ? v0 : -v0, any = true;
+    if (cy) s = any ? (cy > 0 ? __fadd_rn(s, v1) : __fsub_rn(s, v1)) : (cy > 0 ? v1 : -v1), any = true;
+    if (cz) s = any ? (cz > 0 ? __fadd_rn(s, v2) : __fsub_rn(s, v2)) : (cz > 0 ? v2 : -v2);
+    return s;
+}
+__device__ __forceinline__ float dot3(float a0, float a1, float a2, float b0, float b1, float b2)
+{
+    return fmaf(a0, b0, fmaf(a1, b1, __fmul_rn(a2, b2)));
+}
+
+// links with a component +1 / -1 along an axis (bit i for link i)
+constexpr unsigned axis_links(const int (&c)[MLBI_Q], int sign)
+{
+    unsigned m = 0u;
+    for (int i = 0; i < MLBI_Q; ++i)
+        if (c[i] == sign) m |= 1u << i;
+    return m;
+}
+constexpr unsigned kPlusX = axis_links(CX, 1), kMinusX = axis_links(CX, -1);
+constexpr unsigned kPlusY = axis_links(CY, 1), kMinusY = axis_links(CY, -1);
+constexpr unsigned kPlusZ = axis_links(CZ, 1), kMinusZ = axis_links(CZ, -1);
+
+// Sites next to a wall run the same unrolled links as the others and only
+// store differently.  (With a loop over the links there, one at a time, the
+// warps at a wall finished long after the others: 97 x 61 x 45 between walls,
+// fused pass 2 + collision 0.058 -> 0.044 ms; 256 x 16^3, half of them channels,
+// 0.310 -> 0.243 ms per step.)  Periodic lattices take a copy without walls:
+// the branch per link costs 7 % of the fused kernel at 128^3.
+template <int S, bool WALLS, class Pops>
+__device__ __forceinline__ void collide_push_w(const mlbi_params &p, int x, int y, int z, long long r,
                                              const Centre<S> &c, const float (&acc)[S][3], const Pops &pops,
                                              float *__restrict__ fout)
 {
@@ -121,25 +156,23 @@ __device__ __forceinline__ void collide_push(const mlbi_params &p, int x, int y,
     for (int a = 0; a < S; ++a) {
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            ueq[a][q] = c.u[a][q] + half * acc[a][q];
-            ub[q] += c.n[a] * ueq[a][q];
+            ueq[a][q] = fmaf(half, acc[a][q], c.u[a][q]);
+            ub[q] = fmaf(c.n[a], ueq[a][q], ub[q]);
         }
         rho += c.n[a];
     }
     const float irho = rho > 0.f ? 1.f / rho : 0.f;
-    ub[0] *= irho; ub[1] *= irho; ub[2] *= irho;
-    const float ubub = ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) ub[q] = __fmul_rn(ub[q], irho);
+    const float ubub = dot3(ub[0], ub[1], ub[2], ub[0], ub[1], ub[2]);
     const float omega = p.omega;
-    // links that wrap around a periodic face move by -+ the extent; sites next
-    // to a wall take the compact bounce-back path
-    const bool wall_site = (p.wall_axis == 0 && (x == 0 || x == p.nx - 1)) ||
-                           (p.wall_axis == 1 && (y == 0 || y == p.ny - 1)) ||
-                           (p.wall_axis == 2 && (z == 0 || z == p.nz - 1));
     // target site of every moving link (32-bit: the lattice has fewer than
-    // 2^31 sites), the same for every species: tgt[i - 1] for link i
+    // 2^31 sites), the same for every species: tgt[i - 1] for link i; links that
+    // wrap around a periodic face move by -+ the extent
     int tgt[MLBI_Q - 1];
-    if (!wall_site) {
-        const int sy = p.nx, sz = p.nx * p.ny, r32 = (int)r;
+    const int r32 = (int)r;
+    {
+        const int sy = p.nx, sz = p.nx * p.ny;
         const int wxm = x == 0 ? p.nx : 0, wxp = x == p.nx - 1 ? -p.nx : 0;
         const int wym = y == 0 ? sz : 0, wyp = y == p.ny - 1 ? -sz : 0;
         const int wzm = z == 0 ? (int)N : 0, wzp = z == p.nz - 1 ? -(int)N : 0;
@@ -157,6 +190,15 @@ __device__ __forceinline__ void collide_push(const mlbi_params &p, int x, int y,
             tgt[i] = r32 + dm;
         }
     }
+    // bit i set: link i leaves through the low / high wall and bounces back
+    unsigned lo = 0u, hi = 0u;
+    if constexpr (WALLS) {
+        const int at = p.wall_axis == 0 ? x : (p.wall_axis == 1 ? y : z);
+        const int last = (p.wall_axis == 0 ? p.nx : (p.wall_axis == 1 ? p.ny : p.nz)) - 1;
+        if (at == 0) lo = p.wall_axis == 0 ? kMinusX : (p.wall_axis == 1 ? kMinusY : kMinusZ);
+        if (at == last) hi = p.wall_axis == 0 ? kPlusX : (p.wall_axis == 1 ? kPlusY : kPlusZ);
+    }
+    const bool wall_site = WALLS && (lo | hi) != 0u;
 #pragma unroll
     for (int a = 0; a < S; ++a) {
         const float na = c.n[a], dna = c.dn[a];
@@ -166,55 +208,56 @@ __device__ __forceinline__ void collide_push(const mlbi_params &p, int x, int y,
         for (int i = 0; i < MLBI_Q; ++i) fi[i] = pops(a, i);
         const float ua0 = ueq[a][0], ua1 = ueq[a][1], ua2 = ueq[a][2];
         const float a0 = acc[a][0], a1 = acc[a][1], a2 = acc[a][2];
-        const float trM = 2.f * (ua0 * ub[0] + ua1 * ub[1] + ua2 * ub[2]) - ubub;   // tr(ua u + u ua - u u)
-        const float trS = 2.f * (ub[0] * a0 + ub[1] * a1 + ub[2] * a2);             // tr(u a + a u)
-        const float ks = p.src_scale * na;
-        if (!wall_site) {
-            // psi_perp and the forcing split into parts even and odd in c_i:
-            // direction i and its opposite share the even part and flip the odd one.
-            // (Collecting the Hermite-2 terms into one quadratic form per species
-            // saves arithmetic but doubles the FP32 velocity error at 500 steps
-            // against the FP64 oracle: this order is kept.)
-            const float om1 = 1.f - omega;
-            const float K1 = dna - 1.5f * na * trM;          // even part of psi at c = 0
-            const float K2 = -1.5f * ks * trS;                // even part of the forcing at c = 0
-            oa[r] = om1 * fi[0] + WQ[0] * (omega * K1 + K2);
+        const float trM = fmaf(2.f, dot3(ua0, ua1, ua2, ub[0], ub[1], ub[2]), -ubub);   // tr(ua u + u ua - u u)
+        const float trS = 2.f * dot3(ub[0], ub[1], ub[2], a0, a1, a2);                   // tr(u a + a u)
+        const float ks = __fmul_rn(p.src_scale, na);
+        // psi_perp and the forcing split into parts even and odd in c_i:
+        // direction i and its opposite share the even part and flip the odd one.
+        // (Collecting the Hermite-2 terms into one quadratic form per species
+        // saves arithmetic but doubles the FP32 velocity error at 500 steps
+        // against the FP64 oracle: this order is kept.)
+        const float om1 = 1.f - omega;
+        const float K1 = fmaf(__fmul_rn(-1.5f, na), trM, dna);          // even part of psi at c = 0
+        const float K2 = __fmul_rn(__fmul_rn(-1.5f, ks), trS);          // even part of the forcing at c = 0
+        const float n45 = __fmul_rn(4.5f, na), k9 = __fmul_rn(9.f, ks);
+        const float n3 = __fmul_rn(__fmul_rn(3.f, omega), na), k3 = __fmul_rn(3.f, ks);
+        oa[r] = fmaf(om1, fi[0], __fmul_rn(WQ[0], fmaf(omega, K1, K2)));
 #pragma unroll
-            for (int i = 1; i < MLBI_Q; i += 2) {
-                const float cu = CX[i] * ua0 + CY[i] * ua1 + CZ[i] * ua2;
-                const float cb = CX[i] * ub[0] + CY[i] * ub[1] + CZ[i] * ub[2];
-                const float ca = CX[i] * a0 + CY[i] * a1 + CZ[i] * a2;
-                const float even = omega * (K1 + 4.5f * na * (2.f * cu * cb - cb * cb)) + (K2 + 9.f * ks * cb * ca);
-                const float odd = 3.f * (omega * na * cu + ks * ca);
-                (oa + i * N)[tgt[i - 1]] = om1 * fi[i] + WQ[i] * (even + odd);
-                (oa + (i + 1) * N)[tgt[i]] = om1 * fi[i + 1] + WQ[i] * (even - odd);
-            }
-        } else {
-#pragma unroll 1
-            for (int i = 0; i < MLBI_Q; ++i) {
-                const int cx = CXv(i), cy = CYv(i), cz = CZv(i);
-                const float w = WQv(i);
-                const float cu = cx * ua0 + cy * ua1 + cz * ua2;
-                const float cb = cx * ub[0] + cy * ub[1] + cz * ub[2];
-                const float ca = cx * a0 + cy * a1 + cz * a2;
-                const float psi = w * (dna + na * (3.f * cu + 4.5f * (2.f * cu * cb - cb * cb) - 1.5f * trM));
-                const float src = w * ks * (3.f * ca + 9.f * cb * ca - 1.5f * trS);
-                const float fv = pops(a, i);
-                const float post = fv - omega * (fv - psi) + src;
-                const long long q = neighbour(p, x, y, z, cx, cy, cz);
-                if (q >= 0) {
-                    oa[i * N + q] = post;
-                } else {
-                    const int ax = p.wall_axis;
-                    const int cax = ax == 0 ? cx : (ax == 1 ? cy : cz);
-                    const int xa = ax == 0 ? x : (ax == 1 ? y : z);
-                    const float *uw = (xa + cax < 0) ? p.wall_lo : p.wall_hi;
-                    const float cuw = cx * uw[0] + cy * uw[1] + cz * uw[2];
-                    oa[opposite(i) * N + r] = post - 6.f * w * na * cuw;
-                }
+        for (int i = 1; i < MLBI_Q; i += 2) {
+            const float cu = cdot(CX[i], CY[i], CZ[i], ua0, ua1, ua2);
+            const float cb = cdot(CX[i], CY[i], CZ[i], ub[0], ub[1], ub[2]);
+            const float ca = cdot(CX[i], CY[i], CZ[i], a0, a1, a2);
+            const float psi = fmaf(n45, __fmul_rn(cb, fmaf(2.f, cu, -cb)), K1);
+            const float even = fmaf(omega, psi, fmaf(__fmul_rn(k9, cb), ca, K2));
+            const float odd = fmaf(n3, cu, __fmul_rn(k3, ca));
+            const float fp = fmaf(om1, fi[i], __fmul_rn(WQ[i], __fadd_rn(even, odd)));
+            const float fm = fmaf(om1, fi[i + 1], __fmul_rn(WQ[i], __fsub_rn(even, odd)));
+            if (!wall_site) {
+                (oa + i * N)[tgt[i - 1]] = fp;
+                (oa + (i + 1) * N)[tgt[i]] = fm;
+            } else {
+                // halfway bounce-back: a link through a wall comes back as its
+                // opposite, i + 1 for i and i for i + 1, with the wall's velocity
+                const bool pl = (lo >> i) & 1u, ph = (hi >> i) & 1u, ml = (lo >> (i + 1)) & 1u, mh = (hi >> (i + 1)) & 1u;
+                const float wn = __fmul_rn(6.f * WQ[i], na);
+                const float cl = cdot(CX[i], CY[i], CZ[i], p.wall_lo[0], p.wall_lo[1], p.wall_lo[2]);
+                const float ch = cdot(CX[i], CY[i], CZ[i], p.wall_hi[0], p.wall_hi[1], p.wall_hi[2]);
+                if (pl || ph) (oa + (i + 1) * N)[r] = fmaf(-wn, pl ? cl : ch, fp);
+                else (oa + i * N)[tgt[i - 1]] = fp;
+                if (ml || mh) (oa + i * N)[r] = fmaf(wn, ml ? cl : ch, fm);
+                else (oa + (i + 1) * N)[tgt[i]] = fm;
             }
         }
     }
+}
+
+template <int S, class Pops>
+__device__ __forceinline__ void collide_push(const mlbi_params &p, int x, int y, int z, long long r,
+                                             const Centre<S> &c, const float (&acc)[S][3], const Pops &pops,
+                                             float *__restrict__ fout)
+{
+    if (p.wall_axis < 0) collide_push_w<S, false>(p, x, y, z, r, c, acc, pops, fout);
+    else collide_push_w<S, true>(p, x, y, z, r, c, acc, pops, fout);
 }
 
 }  // namespace

@@ -16,19 +16,6 @@ __device__ constexpr float WQ[MLBI_Q] = {1.f / 3.f,
                                          1.f / 36.f, 1.f / 36.f, 1.f / 36.f, 1.f / 36.f, 1.f / 36.f, 1.f / 36.f,
                                          1.f / 36.f, 1.f / 36.f, 1.f / 36.f, 1.f / 36.f, 1.f / 36.f, 1.f / 36.f};
 
-__device__ __forceinline__ int opposite(int i) { return i == 0 ? 0 : (((i - 1) ^ 1) + 1); }
-
-// the same velocity set for a runtime index, from bit tables (no memory access):
-// component = (bit of "plus" mask) - (bit of "minus" mask)
-__device__ __forceinline__ int comp_of(int i, unsigned plus, unsigned minus)
-{
-    return (int)((plus >> i) & 1u) - (int)((minus >> i) & 1u);
-}
-__device__ __forceinline__ int CXv(int i) { return comp_of(i, 0x2A82u, 0x5504u); }
-__device__ __forceinline__ int CYv(int i) { return comp_of(i, 0x28488u, 0x50310u); }
-__device__ __forceinline__ int CZv(int i) { return comp_of(i, 0x4C820u, 0x33040u); }
-__device__ __forceinline__ float WQv(int i) { return i == 0 ? 1.f / 3.f : (i < 7 ? 1.f / 18.f : 1.f / 36.f); }
-
 constexpr int kBlock = 256;
 constexpr float kTinyDensity = 1e-12f;
 

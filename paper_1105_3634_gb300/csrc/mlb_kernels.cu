@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kBlock) k_moments_g_group(const mlbi_member *_
 }
 
 template <int S>
-__global__ void __launch_bounds__(kBX * kBY, 6) k_collide(const mlbi_params p, const float *__restrict__ fin,
+__global__ void __launch_bounds__(kBX * kBY, 5) k_collide(const mlbi_params p, const float *__restrict__ fin,
                                                           float *__restrict__ fout, const float4 *__restrict__ mom,
                                                           const float4 *__restrict__ accf)
 {

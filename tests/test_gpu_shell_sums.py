@@ -92,3 +92,33 @@ def test_narrow_tiles(gpu, orc, name):
         out.append(sim.populations()[0])
         sim.close()
     assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
+
+
+# rows that are no multiple of 16 bytes, walls on every axis (one site thick too)
+ROWS = {
+    "one_over": dict(sigma=[1.0, 1.5], shape=(33, 5, 7)),
+    "two_over": dict(sigma=[1.0, 1.5], shape=(34, 8, 3), wall_axis=0),
+    "narrow": dict(sigma=[1.0, 1.5], shape=(17, 9, 6), wall_axis=1),
+    "three_short": dict(sigma=[1.0], shape=(61, 3, 5)),
+    "one_plane": dict(sigma=[1.0, 1.5], shape=(18, 7, 1), wall_axis=2, wall_u_lo=(0.01, 0.0, 0.0),
+                      wall_u_hi=(0.0, 0.02, 0.0)),
+    "moving_x": dict(sigma=[1.0, 1.5], shape=(20, 7, 6), wall_axis=0, wall_u_lo=(0.0, 0.02, -0.01),
+                     wall_u_hi=(0.0, -0.01, 0.02)),
+    "reach2": dict(sigma=[1.5, 2.0], shape=(35, 6, 9), drag_only=True),
+    "three_species": dict(sigma=[1.0, 1.25, 1.5], shape=(37, 5, 6), wall_axis=2),
+}
+
+
+@pytest.mark.parametrize("name", sorted(ROWS))
+def test_unaligned_rows(gpu, orc, name):
+    lat = W.Lattice(**ROWS[name])
+    n, u = fields(lat, 0.1)
+    check(gpu, orc, lat, n, u, 3)
+    out = []
+    for split in (False, True):
+        sim = gpu.Simulation(lat, split_collide=split)
+        sim.set_fields(n, u)
+        sim.step(4)
+        out.append(sim.populations()[0])
+        sim.close()
+    assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
