@@ -312,7 +312,6 @@ mlb_status rebuild(mlb_ctx *c)
             shell_reach = std::max(shell_reach, (int)std::floor(std::sqrt(std::pow(sab + 0.5, 2) - 1e-9)));
         }
     const int tile_r = mlbi_tile_ty(S, shell_reach) ? shell_reach : 0;
-    const int txh = 32 + 2 * tile_r;
     // reach of the attraction regions (column attraction kernel if <= 8)
     int attr_reach = 0;
     for (int a = 0; a < S; ++a)
@@ -328,16 +327,25 @@ mlb_status rebuild(mlb_ctx *c)
         std::memcpy(&e0.w, &packed, sizeof(int));
         long long lin = dx + nx * dy + nxy * dz;
         if (lin >= (1ll << 31) || lin <= -(1ll << 31)) lin_overflow = true;
-        int lin32 = (int)lin, tileoff = dx + txh * dy, dzz = dz;
+        int lin32 = (int)lin, zero = 0;
         std::memcpy(&e1.x, &lin32, sizeof(int));
         std::memcpy(&e1.y, &mask, sizeof(int));
-        std::memcpy(&e1.z, &tileoff, sizeof(int));
-        std::memcpy(&e1.w, &dzz, sizeof(int));
+        std::memcpy(&e1.z, &zero, sizeof(int));
+        std::memcpy(&e1.w, &zero, sizeof(int));
         tab.push_back(e0);
         tab.push_back(e1);
         maxoff = std::max(maxoff, std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))));
     };
     auto count = [&]() { return (int)(tab.size() / 2); };
+    // an offset of a contact shell: the kernels read sign groups, the bounds on
+    // offsets and on the shells' size hold for every offset
+    size_t shell_offsets = 0;
+    auto note = [&](int dx, int dy, int dz) {
+        const long long lin = dx + nx * dy + nxy * dz;
+        if (lin >= (1ll << 31) || lin <= -(1ll << 31)) lin_overflow = true;
+        maxoff = std::max(maxoff, std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))));
+        ++shell_offsets;
+    };
     // smoothing balls |d| <= kappa sigma_c (origin included)
     for (int g = 0; g < S; ++g) {
         double R = c->desc.kappa * c->sigma[g];
@@ -367,16 +375,15 @@ mlb_status rebuild(mlb_ctx *c)
             mlbi_pair &pr = p.pair[np];
             const double sab = 0.5 * (c->sigma[a] + c->sigma[b]);
             const int Ri = (int)std::ceil(sab + 0.5) + 1;
-            pr.shell_start = count();
+            int shell_count = 0;
             for (int dz = -Ri; dz <= Ri; ++dz)
                 for (int dy = -Ri; dy <= Ri; ++dy)
-                    for (int dx = -Ri; dx <= Ri; ++dx) {
-                        if (!canonical(dx, dy, dz) || !in_shell(sab, dx, dy, dz)) continue;
-                        const double len = std::sqrt((double)(dx * dx + dy * dy + dz * dz));
-                        push(dx, dy, dz, dx / len, dy / len, dz / len, 0);
-                    }
-            pr.shell_count = count() - pr.shell_start;
-            const double wS = 4.0 * kPi / (2.0 * pr.shell_count);
+                    for (int dx = -Ri; dx <= Ri; ++dx)
+                        if (canonical(dx, dy, dz) && in_shell(sab, dx, dy, dz)) {
+                            note(dx, dy, dz);
+                            ++shell_count;
+                        }
+            const double wS = 4.0 * kPi / (2.0 * shell_count);
             const double mu = c->mass[a] * c->mass[b] / (c->mass[a] + c->mass[b]);
             pr.hc_pre = (float)(c->desc.kT * sab * sab * wS);
             pr.vx_pre = (float)(2.0 * sab * sab * std::sqrt(2.0 * mu * c->desc.kT / kPi) * wS);
@@ -405,24 +412,39 @@ mlb_status rebuild(mlb_ctx *c)
             p.pair_index[a][b] = p.pair_index[b][a] = np;
             ++np;
         }
-    // union half shells per neighbour species b, with a mask of the species a
-    // whose pair shell (a, b) contains the offset
+    // union half shells per neighbour species b as sign groups (mlb_groups.cuh), by type,
+    // with a mask of the species a whose pair shell (a, b) contains the length
+    p.grp_at = (int)tab.size();
+    int ngroups = 0;
     for (int b = 0; b < S; ++b) {
         int R = 1;
         for (int a = 0; a < S; ++a) R = std::max(R, (int)std::ceil(0.5 * (c->sigma[a] + c->sigma[b]) + 0.5) + 1);
-        p.ushell_start[b] = count();
-        for (int dz = -R; dz <= R; ++dz)
-            for (int dy = -R; dy <= R; ++dy)
-                for (int dx = -R; dx <= R; ++dx) {
-                    if (!canonical(dx, dy, dz)) continue;
-                    int mask = 0;
-                    for (int a = 0; a < S; ++a)
-                        if (in_shell(0.5 * (c->sigma[a] + c->sigma[b]), dx, dy, dz)) mask |= 1 << a;
-                    if (!mask) continue;
-                    const double len = std::sqrt((double)(dx * dx + dy * dy + dz * dz));
-                    push(dx, dy, dz, dx / len, dy / len, dz / len, mask);
-                }
-        p.ushell_count[b] = count() - p.ushell_start[b];
+        for (int type = 0; type < 7; ++type) {
+            p.grp[b][type] = ngroups;
+            // which of X, Y, Z are non-zero, as in mlb_groups.cuh
+            const int has = type < 3 ? 1 << type : (type == 3 ? 3 : (type == 4 ? 5 : (type == 5 ? 6 : 7)));
+            for (int Z = (has & 4) ? 1 : 0; Z <= ((has & 4) ? R : 0); ++Z)
+                for (int Y = (has & 2) ? 1 : 0; Y <= ((has & 2) ? R : 0); ++Y)
+                    for (int X = (has & 1) ? 1 : 0; X <= ((has & 1) ? R : 0); ++X) {
+                        int mask = 0;
+                        for (int a = 0; a < S; ++a)
+                            if (in_shell(0.5 * (c->sigma[a] + c->sigma[b]), X, Y, Z)) mask |= 1 << a;
+                        if (!mask) continue;
+                        shell_offsets += type < 3 ? 1 : (type < 6 ? 2 : 4);
+                        const double len = std::sqrt((double)(X * X + Y * Y + Z * Z));
+                        mlbi_entry e0, e1;
+                        e0.x = (float)(X / len); e0.y = (float)(Y / len); e0.z = (float)(Z / len);
+                        std::memcpy(&e0.w, &mask, sizeof(int));
+                        std::memcpy(&e1.x, &X, sizeof(int));
+                        std::memcpy(&e1.y, &Y, sizeof(int));
+                        std::memcpy(&e1.z, &Z, sizeof(int));
+                        e1.w = 0.f;
+                        tab.push_back(e0);
+                        tab.push_back(e1);
+                        ++ngroups;
+                    }
+        }
+        p.grp[b][7] = ngroups;
     }
     if (attraction) maxoff = std::max(maxoff, attr_reach);
     // column form of the attraction: the region sigma_ab <= |d| <= lambda_c sigma_ab
@@ -483,9 +505,12 @@ mlb_status rebuild(mlb_ctx *c)
         }
     }
     if (lin_overflow) return fail(c, MLB_EINVAL, "stencil offsets exceed 32-bit linear offsets on this lattice");
-    if (tab.size() > 2 * (size_t)kTableCap)
+    // the capacity counts every shell offset (two float4) as well as the tables;
+    // the groups' entries, fewer than their offsets, are within it
+    const size_t need = tab.size() - 2 * (size_t)ngroups + 2 * shell_offsets;
+    if (need > 2 * (size_t)kTableCap)
         return fail(c, MLB_EINVAL, "stencil tables need %d float4, capacity is %d (reduce sigma or lambda_c)",
-                    (int)tab.size(), 2 * kTableCap);
+                    (int)need, 2 * kTableCap);
     const int L[3] = {c->desc.nx, c->desc.ny, c->desc.nz};
     for (int ax = 0; ax < 3; ++ax)
         if (ax != c->desc.wall_axis && L[ax] <= maxoff)

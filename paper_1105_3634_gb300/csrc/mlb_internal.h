@@ -14,11 +14,7 @@
 // One stencil entry is two float4 in the table:
 //   e0 = (x, y, z, packed d): a unit vector s_d or a kernel vector, and the
 //        offset d packed as three signed 10-bit fields (see mlbi_pack);
-//   e1 = (linear offset of d for this lattice, mask, tile offset, dz) as
-//        int bits; the mask (union shells) has bit a set when d lies in the
-//        shell of the pair (a, b) of the table's neighbour species b; the
-//        tile offset dx + dy (32 + 2 tile_r) addresses d inside a plane of
-//        the shared-memory tile of the tiled kernels.
+//   e1 = (linear offset of d for this lattice as int bits, 0, 0, 0).
 typedef float4 mlbi_entry;
 
 __host__ __device__ inline int mlbi_pack(int dx, int dy, int dz)
@@ -33,7 +29,6 @@ __host__ __device__ inline void mlbi_unpack(int p, int &dx, int &dy, int &dz)
 }
 
 struct mlbi_pair {               // unordered pair a <= b, index a*S - a(a-1)/2 + (b - a)
-    int shell_start, shell_count;    // half shell: one of each +-d (entries)
     int attr_start, attr_count;      // half attraction region (entries)
     float hc_pre;                    // kT sigma_ab^2 4 pi / |S_ab|
     float vx_pre;                    // K_ab 4 pi / |S_ab|,  K_ab = 2 sigma_ab^2 sqrt(2 mu_ab kT / pi)
@@ -58,10 +53,13 @@ struct mlbi_params {
     float xi2_ref, xi3_ref;
     int ball_start[MLBI_MAXS], ball_count[MLBI_MAXS];
     float ball_inv[MLBI_MAXS];
-    int ushell_start[MLBI_MAXS], ushell_count[MLBI_MAXS];   // union half shells per neighbour species
     int reach;                       // largest offset component of any stencil (>= 1)
     int local_g;                     // every smoothing ball is the single site
     int tile_r;                      // reach of the union shells if the tiled kernels serve it (1..3), else 0
+    // sign groups of the union half shells (mlb_groups.cuh), two float4 each from
+    // table[grp_at]: (|s_x|, |s_y|, |s_z|, mask of the species a), (X, Y, Z, 0);
+    // grp[b][t] the first of type t for neighbour species b, grp[b][7] the end
+    int grp_at, grp[MLBI_MAXS][8];
     int cube_mask[MLBI_MAXP];        // tile_r == 1: bit k set when half offset k of the 3x3x3 cube is in S_ab
     int attr_r;                      // reach of the attraction if the column attraction kernel serves it (1..8), else 0
     // column form of the attraction (attr_r > 0): acol_count columns (dx, dy) of the
@@ -78,32 +76,24 @@ struct mlbi_params {
 };
 
 // Shared-memory z-marching tiles of the stencil passes: a ring of 2R + 2
-// planes of (32 + 2R) x (ty + 2R) sites, each site S float4 fields and
-// S(S+1)/2 contact-value deviations.  Tiles serve shell reach R <= 3; reach 1
-// and 2 use 32 x 4 blocks, reach 3 32 x 8 blocks where they fit, else 32 x 4.
+// planes of (tx + 2R) x (ty + 2R) sites, each site S float4 fields and
+// S(S+1)/2 contact-value deviations.  Reach 3 tiles leave room for one block
+// per SM, so `split` threads share a site there (each takes every split-th
+// group of the shell table) to keep enough warps resident; their partial sums
+// meet in shared memory behind the ring.
 #define MLBI_MAX_TILE_BYTES (227 * 1024)
-__host__ __device__ constexpr long long mlbi_tile_bytes(int S, int R, int ty)
+struct mlbi_tile {
+    int tx, ty, split;               // ty = 0: no tile, the global-memory passes
+};
+__host__ __device__ constexpr mlbi_tile mlbi_tile_of(int S, int R)
 {
-    return (long long)(2 * R + 2) * (32 + 2 * R) * (ty + 2 * R) * (S * 16 + S * (S + 1) / 2 * 4);
+    return R == 1 ? mlbi_tile{32, 4, 1}
+         : R == 2 ? mlbi_tile{32, 4, S == 3 ? 3 : 2}
+         : R == 3 && S <= 2 ? mlbi_tile{32, 8, 2}
+         : R == 3 && S == 3 ? mlbi_tile{16, 8, 3}
+         : mlbi_tile{32, 0, 1};
 }
-// warps per SM that tiles of block height ty leave resident (the shared-memory
-// bound: 228 KB per SM, 1 KB reserved per block)
-__host__ __device__ constexpr long long mlbi_tile_warps(int S, int R, int ty)
-{
-    return (228 * 1024) / (mlbi_tile_bytes(S, R, ty) + 1024) * ty;
-}
-// block height of the tile for (S, R), or 0 for the global-memory passes: a
-// tile that fits and leaves at least 8 resident warps per SM (one 4-warp
-// block per SM is latency-bound: measured slower than the global passes for
-// three species at reach 3, while one 8-warp block per SM beats them for
-// two species at reach 3)
-__host__ __device__ constexpr int mlbi_tile_ty(int S, int R)
-{
-    return R < 1 || R > 3 ? 0
-         : R < 3 ? (mlbi_tile_bytes(S, R, 4) <= MLBI_MAX_TILE_BYTES && mlbi_tile_warps(S, R, 4) >= 8 ? 4 : 0)
-         : mlbi_tile_bytes(S, R, 8) <= MLBI_MAX_TILE_BYTES ? 8
-         : (mlbi_tile_bytes(S, R, 4) <= MLBI_MAX_TILE_BYTES && mlbi_tile_warps(S, R, 4) >= 8 ? 4 : 0);
-}
+__host__ __device__ constexpr int mlbi_tile_ty(int S, int R) { return mlbi_tile_of(S, R).ty; }
 
 // ------------------------------------------------------------------ work decomposition of the tiled passes
 // Tile width of the reach-1 passes (one and two species): 32 x 4 sites, or 16
@@ -124,11 +114,13 @@ inline int mlbi_tile_x(int S, int tile_r, int nx, int ny)
 }
 // rows of a tile of pass 1 and of the fused pass 2 + collision
 inline int mlbi_tile_rows(const mlbi_params &p) { return p.tile_r == 1 ? 128 / p.tile_x : mlbi_tile_ty(p.S, p.tile_r); }
+inline int mlbi_tile_cols(const mlbi_params &p) { return p.tile_r == 1 ? p.tile_x : mlbi_tile_of(p.S, p.tile_r).tx; }
 // tile planes (one tile of one z plane) of a lattice
 inline long long mlbi_tile_planes(const mlbi_params &p)
 {
     const int ty = mlbi_tile_rows(p);
-    return ty < 1 ? 0 : (long long)((p.nx + p.tile_x - 1) / p.tile_x) * ((p.ny + ty - 1) / ty) * p.nz;
+    const int tx = mlbi_tile_cols(p);
+    return ty < 1 ? 0 : (long long)((p.nx + tx - 1) / tx) * ((p.ny + ty - 1) / ty) * p.nz;
 }
 // Planes per block.  A block pays about one plane's time for filling its ring,
 // and the kernel's last blocks run about one block's time with the GPU
@@ -237,6 +229,27 @@ cudaError_t mlbi_launch_collide(const mlbi_params &p, const mlbi_buffers &b, int
 // in shared memory), else cudaErrorInvalidValue
 bool mlbi_pass2_collide_supported(const mlbi_params &p);
 cudaError_t mlbi_launch_pass2_collide(const mlbi_params &p, const mlbi_buffers &b, int cur, cudaStream_t s);
+// the passes by species count (one compilation unit per count above two)
+template <int S> cudaError_t mlbi_pass1_species(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s);
+template <> cudaError_t mlbi_pass1_species<1>(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s);
+template <> cudaError_t mlbi_pass1_species<2>(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s);
+template <> cudaError_t mlbi_pass1_species<3>(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s);
+template <> cudaError_t mlbi_pass1_species<4>(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s);
+template <int S> cudaError_t mlbi_sweep_species(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next, cudaStream_t s);
+template <> cudaError_t mlbi_sweep_species<1>(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next, cudaStream_t s);
+template <> cudaError_t mlbi_sweep_species<2>(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next, cudaStream_t s);
+template <> cudaError_t mlbi_sweep_species<3>(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next, cudaStream_t s);
+template <> cudaError_t mlbi_sweep_species<4>(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next, cudaStream_t s);
+template <int S> cudaError_t mlbi_pass2_species(const mlbi_params &p, const mlbi_buffers &b, double *acc_out, cudaStream_t s);
+template <> cudaError_t mlbi_pass2_species<1>(const mlbi_params &p, const mlbi_buffers &b, double *acc_out, cudaStream_t s);
+template <> cudaError_t mlbi_pass2_species<2>(const mlbi_params &p, const mlbi_buffers &b, double *acc_out, cudaStream_t s);
+template <> cudaError_t mlbi_pass2_species<3>(const mlbi_params &p, const mlbi_buffers &b, double *acc_out, cudaStream_t s);
+template <> cudaError_t mlbi_pass2_species<4>(const mlbi_params &p, const mlbi_buffers &b, double *acc_out, cudaStream_t s);
+template <int S> cudaError_t mlbi_pass2_collide_species(const mlbi_params &p, const mlbi_buffers &b, int cur, cudaStream_t s);
+template <> cudaError_t mlbi_pass2_collide_species<1>(const mlbi_params &p, const mlbi_buffers &b, int cur, cudaStream_t s);
+template <> cudaError_t mlbi_pass2_collide_species<2>(const mlbi_params &p, const mlbi_buffers &b, int cur, cudaStream_t s);
+template <> cudaError_t mlbi_pass2_collide_species<3>(const mlbi_params &p, const mlbi_buffers &b, int cur, cudaStream_t s);
+template <> cudaError_t mlbi_pass2_collide_species<4>(const mlbi_params &p, const mlbi_buffers &b, int cur, cudaStream_t s);
 cudaError_t mlbi_launch_init(const mlbi_params &p, const mlbi_buffers &b, int cur, const double *n,
                              const double *u, cudaStream_t s);
 cudaError_t mlbi_launch_export_moments(const mlbi_params &p, const mlbi_buffers &b, double *n_out,

@@ -2,9 +2,9 @@
 // hard-core force (Eq. potmeanforce), the velocity exchange (Eqs. gammaab,
 // viscousforce) at u, the friction matrix Gamma^a, the attraction read-in,
 // and the half-step predictor du of the semi-implicit forcing.  Three
-// variants of the shell sums: global-memory (any reach), shared-memory tile
-// with the stencil table (reach 2, 3), and the compile-time 3x3x3 cube
-// (reach 1).  The kernels come in three modes:
+// variants of the shell sums: global memory with the sign groups (any reach),
+// shared-memory tile with the sign groups (reach 2, 3), and the compile-time
+// 3x3x3 cube (reach 1).  The kernels come in three modes:
 //   kExact      the method's pass 1 (mlb_pass1.cu)
 //   kSurrogate  F^hc taken from attr (the learned surrogate's), no hard-core sums
 //   kSweep      a further Jacobi sweep of the half step u* = u + a(u*)/2: the
@@ -16,6 +16,7 @@
 
 #include "mlb_passes.cuh"
 #include "mlb_cube.cuh"
+#include "mlb_groups.cuh"
 
 namespace {
 
@@ -56,52 +57,55 @@ struct Acc1 {
             }
         }
     }
-};
-
-// Shell sums from global memory, for every species a over neighbour species b:
-//   hard core  -hc_ab sum_{+-d} s (g(r)+g(r+d))/2 n^b(r+d)                          (Eq. potmeanforce)
-//   exchange   vx_ab sum_{+-d} s s.[(g(r)+g(r+d))/2 n^b(r+d) (u^b(r+d) - u^a(r))]  (Eqs. gammaab, viscousforce)
-//   friction   Gamma^a = vx_ab sum_{+-d} s s^T (g(r)+g(r+d))/2 n^b(r+d)
-template <int S, bool DRAG, bool INTERIOR, bool HC>
-__device__ __forceinline__ void pass1_shells(const mlbi_params &p, const Loc &L, const Centre<S> &c,
-                                             const float (&ub)[S][3], const PairW<S> &w,
-                                             const float4 *__restrict__ mom, const float *__restrict__ dg,
-                                             const mlbi_entry *__restrict__ tab, Acc1<S> &A)
-{
-    const long long N = p.N;
+    // the shell sums of (a, b): D hard core, E = sum s s^T (W+ + W-), J the
+    // exchange relative to the partners' velocity u^b(r), completed by
+    // Gamma_ab w, w = u^b(r) - u^a(r) (drag); K = vx_ab / 2, H = -hc_ab / 2
+    template <bool DRAG, bool HC>
+    __device__ __forceinline__ void add(int a, float K, float H, const float (&D)[3], const float (&E)[6],
+                                        const float (&J)[3], const float (&w)[3], bool drag)
+    {
+        float e[6];
 #pragma unroll
-    for (int b = 0; b < S; ++b) {
-        const int k0 = p.ushell_start[b], k1 = k0 + p.ushell_count[b];
-        const float4 *fb = mom + b * N;
-#pragma unroll 2
-        for (int k = k0; k < k1; ++k) {
-            const float4 e0 = __ldg(&tab[2 * k]);
-            const float4 e1 = __ldg(&tab[2 * k + 1]);
-            const int mask = __float_as_int(e1.y);
-            const Nb P = fetch_nb<INTERIOR>(p, L, e0, e1, 1, fb, p.nref[b]);
-            const Nb M = fetch_nb<INTERIOR>(p, L, e0, e1, -1, fb, p.nref[b]);
-            const float sx = e0.x, sy = e0.y, sz = e0.z;
-            const float jp = DRAG ? 0.f : sx * P.u0 + sy * P.u1 + sz * P.u2;
-            const float jm = DRAG ? 0.f : sx * M.u0 + sy * M.u1 + sz * M.u2;
+        for (int k = 0; k < 6; ++k) e[k] = K * E[k];
+        G[a][0] = add2(G[a][0], f2(e[0], e[1]));
+        G[a][1] = add2(G[a][1], f2(e[2], e[3]));
+        G[a][2] = add2(G[a][2], f2(e[4], e[5]));
+        if constexpr (HC)
 #pragma unroll
-            for (int a = 0; a < S; ++a) {
-                if (!(mask & (1 << a))) continue;
-                const int q = pair_of(a, b, S);
-                const float su = DRAG ? 0.f : sx * c.u[a][0] + sy * c.u[a][1] + sz * c.u[a][2];
-                const float *dgq = dg + q * N;
-                const float dgp = (INTERIOR || P.q >= 0) ? dgq[P.q] : 0.f;
-                const float dgm = (INTERIOR || M.q >= 0) ? dgq[M.q] : 0.f;
-                const float sdu = DRAG ? sx * (c.u[a][0] - ub[b][0]) + sy * (c.u[a][1] - ub[b][1]) +
-                                             sz * (c.u[a][2] - ub[b][2])
-                                       : 0.f;
-                float t, sd, wn;
-                pass1_point<DRAG>(P.n, M.n, P.dn - M.dn, jp - su, jm - su, dgp, dgm, w.kp[q], 0.5f * p.pair[q].vx_pre, w.h[q],
-                                  -0.5f * p.pair[q].hc_pre, sdu, t, sd, wn);
-                add_pass1(sx, sy, sz, HC ? t : 0.f, sd, wn, A.hf[a], A.G[a]);
-            }
+            for (int k = 0; k < 3; ++k) hf[a][k].x = fmaf(H, D[k], hf[a][k].x);
+        if constexpr (!DRAG)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) hf[a][k].y = fmaf(K, J[k], hf[a][k].y);
+        if (drag) {
+            hf[a][0].y = fmaf(e[0], w[0], fmaf(e[3], w[1], fmaf(e[4], w[2], hf[a][0].y)));
+            hf[a][1].y = fmaf(e[3], w[0], fmaf(e[1], w[1], fmaf(e[5], w[2], hf[a][1].y)));
+            hf[a][2].y = fmaf(e[4], w[0], fmaf(e[5], w[1], fmaf(e[2], w[2], hf[a][2].y)));
         }
     }
-}
+    // the 12 partial sums per species of a part, stride n floats apart
+    __device__ __forceinline__ void put(float *m, int n) const
+    {
+#pragma unroll
+        for (int a = 0; a < S; ++a)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                m[(a * 12 + k) * n] = hf[a][k].x;
+                m[(a * 12 + 3 + k) * n] = hf[a][k].y;
+                m[(a * 12 + 6 + k) * n] = G[a][k].x;
+                m[(a * 12 + 9 + k) * n] = G[a][k].y;
+            }
+    }
+    __device__ __forceinline__ void take(const float *m, int n)
+    {
+#pragma unroll
+        for (int a = 0; a < S; ++a)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                hf[a][k] = add2(hf[a][k], f2(m[(a * 12 + k) * n], m[(a * 12 + 3 + k) * n]));
+                G[a][k] = add2(G[a][k], f2(m[(a * 12 + 6 + k) * n], m[(a * 12 + 9 + k) * n]));
+            }
+    }
+};
 
 // attraction sum_{+d} K_ab(d) (n^b(r+d) - n^b(r-d)) from global memory (G term
 // of Eq. potmeanforce, RPA), for reaches the column kernel does not serve
@@ -210,38 +214,53 @@ __device__ __forceinline__ void centre_of(const mlbi_params &p, const float4 (&c
     }
 }
 
+// ------------------------------------------------------------------ global memory
+// Shells beyond the tiles (reach 4 and more; four species at reach 3).  A block
+// takes 32 consecutive sites, each by kParts threads (one warp per part) that
+// share the groups: enough warps for small lattices of large spheres (80 x 40 x
+// 40 has 4000 site warps for 152 SMs), no idle lanes at ragged widths, and the
+// parts read neighbouring rows at the same time.  Measured (sigma = 8 / 4, 925
+// pairs a site, 80 x 40 x 40): pass 1 1.419 -> 0.496 ms, pass 2 1.043 ->
+// 0.437 (one thread per site, a table entry per pair, every neighbour of a site near a
+// face wrapped by itself: three quarters of the sites).
+constexpr int kParts = 4;
+
 template <int S, bool DRAG, int MODE>
-__global__ void __launch_bounds__(kBX * kBY) k_pass1(const mlbi_params p, const float4 *__restrict__ mom,
-                                                     const float *__restrict__ dg,
-                                                     const mlbi_entry *__restrict__ tab,
-                                                     const float4 *__restrict__ fext,
-                                                     const float4 *__restrict__ attr,
-                                                     const float4 *__restrict__ mom_c, float4 *__restrict__ frest,
-                                                     float4 *__restrict__ pst)
+__global__ void __launch_bounds__(32 * kParts, 4) k_pass1(const mlbi_params p, const float4 *__restrict__ mom,
+                                                          const float *__restrict__ dg,
+                                                          const mlbi_entry *__restrict__ tab,
+                                                          const float4 *__restrict__ fext,
+                                                          const float4 *__restrict__ attr,
+                                                          const float4 *__restrict__ mom_c, float4 *__restrict__ frest,
+                                                          float4 *__restrict__ pst)
 {
-    constexpr int NP = S * (S + 1) / 2;
     step_begin();
+    __shared__ float red[kParts - 1][12 * S][32];
+    const long long N = p.N, r = blockIdx.x * 32ll + threadIdx.x;
+    const int part = threadIdx.y;
+    const bool active = r < N;
     Loc L;
-    if (!locate(p, L)) return;
-    const long long N = p.N, r = L.r;
+    L.r = r;
+    L.x = (int)(r % p.nx);
+    L.y = (int)(r / p.nx % p.ny);
+    L.z = (int)(r / ((long long)p.nx * p.ny));
     Centre<S> c;
-    float ub[S][3];
-    {
+    Acc1<S> A;
+    A.zero();
+    if (active) {
+        float ub[S][3];
         float4 cv[S];
 #pragma unroll
         for (int a = 0; a < S; ++a) cv[a] = mom[a * N + r];
         centre_of<S, MODE>(p, cv, mom_c, r, c, ub);
+        const GlobalView<S> view{p, mom, dg, L.x, L.y, L.z};
+        p1_groups<S, kParts, DRAG, MODE == kSweep, MODE == kExact>(p, tab + p.grp_at, view, c.u, part, A);
+        if (part > 0) A.put(&red[part - 1][0][threadIdx.x], 32);
     }
-    float dgc[NP];
+    __syncthreads();
+    if (!active || part > 0) return;
 #pragma unroll
-    for (int q = 0; q < NP; ++q) dgc[q] = dg[q * N + r];
-    PairW<S> w;
-    pair_weights<S>(p, dgc, w);
-    Acc1<S> A;
-    A.zero();
-    constexpr bool HC = MODE == kExact;
-    if (L.interior) pass1_shells<S, DRAG, true, HC>(p, L, c, ub, w, mom, dg, tab, A);
-    else pass1_shells<S, DRAG, false, HC>(p, L, c, ub, w, mom, dg, tab, A);
+    for (int k = 0; k < kParts - 1; ++k) A.take(&red[k][0][threadIdx.x], 32);
     if constexpr (MODE == kSweep) {
         sweep_finish<S>(p, r, c, A, frest, pst);
         return;
@@ -253,6 +272,8 @@ __global__ void __launch_bounds__(kBX * kBY) k_pass1(const mlbi_params p, const 
             A.at[a][0] = v.x; A.at[a][1] = v.y; A.at[a][2] = v.z;
         }
     } else if (p.has_attraction) {
+        const int R = p.reach;
+        L.interior = L.x >= R && L.x < p.nx - R && L.y >= R && L.y < p.ny - R && L.z >= R && L.z < p.nz - R;
         if (L.interior) pass1_attraction<S, true>(p, L, mom, tab, A.at);
         else pass1_attraction<S, false>(p, L, mom, tab, A.at);
     }
@@ -260,49 +281,6 @@ __global__ void __launch_bounds__(kBX * kBY) k_pass1(const mlbi_params p, const 
 }
 
 // ------------------------------------------------------------------ tiled variants
-// Shell sums from the tile with the stencil table (same sums as pass1_shells).
-template <int S, int R, bool DRAG, int TY, bool HC>
-__device__ __forceinline__ void pass1_tile_shells(const mlbi_params &p, const mlbi_entry *tab,
-                                                  const float4 *sf, const float *sg, int kz, int cidx,
-                                                  const Centre<S> &c, const float (&ub)[S][3], const PairW<S> &w,
-                                                  Acc1<S> &A)
-{
-    using T = Tile<S, R, TY>;
-#pragma unroll
-    for (int b = 0; b < S; ++b) {
-        const float nr = p.nref[b];
-        const int k0 = p.ushell_start[b], k1 = k0 + p.ushell_count[b];
-#pragma unroll 2
-        for (int k = k0; k < k1; ++k) {
-            const float4 e0 = tab[2 * k];                   // global or shared (stage_table)
-            const float4 e1 = tab[2 * k + 1];
-            const int mask = __float_as_int(e1.y), off = __float_as_int(e1.z), dz = __float_as_int(e1.w);
-            const int sp = ring(kz + dz, T::NSLOT), sm = ring(kz - dz, T::NSLOT);   // ring slots of the +-d planes
-            const float4 vp = sf[sp * S * T::PLANE + b * T::PLANE + cidx + off];
-            const float4 vm = sf[sm * S * T::PLANE + b * T::PLANE + cidx - off];
-            const float np = nr + vp.x, nm = nr + vm.x, dd = vp.x - vm.x;
-            const float sx = e0.x, sy = e0.y, sz = e0.z;
-            const float jp = DRAG ? 0.f : sx * vp.y + sy * vp.z + sz * vp.w;
-            const float jm = DRAG ? 0.f : sx * vm.y + sy * vm.z + sz * vm.w;
-#pragma unroll
-            for (int a = 0; a < S; ++a) {
-                if (!(mask & (1 << a))) continue;
-                const int q = pair_of(a, b, S);
-                const float su = DRAG ? 0.f : sx * c.u[a][0] + sy * c.u[a][1] + sz * c.u[a][2];
-                const float dgp = sg[sp * T::NP * T::PLANE + q * T::PLANE + cidx + off];
-                const float dgm = sg[sm * T::NP * T::PLANE + q * T::PLANE + cidx - off];
-                const float sdu = DRAG ? sx * (c.u[a][0] - ub[b][0]) + sy * (c.u[a][1] - ub[b][1]) +
-                                             sz * (c.u[a][2] - ub[b][2])
-                                       : 0.f;
-                float t, sd, wn;
-                pass1_point<DRAG>(np, nm, dd, jp - su, jm - su, dgp, dgm, w.kp[q], 0.5f * p.pair[q].vx_pre, w.h[q],
-                                  -0.5f * p.pair[q].hc_pre, sdu, t, sd, wn);
-                add_pass1(sx, sy, sz, HC ? t : 0.f, sd, wn, A.hf[a], A.G[a]);
-            }
-        }
-    }
-}
-
 // Shell sums for reach 1 (mlb_cube.cuh), folded into the site's force sums.
 // The exchange sums are relative to the partners' own velocity at r (ub):
 // Gamma_ab (u^b(r) - u^a(r)) completes them.
@@ -320,25 +298,16 @@ __device__ __forceinline__ void pass1_cube(const mlbi_params &p, const float4 *s
 #pragma unroll
         for (int a = 0; a < S; ++a) {
             const mlbi_pair &pr = p.pair[pair_of(a, b, S)];
-            const float K = 0.5f * pr.vx_pre, H = -0.5f * pr.hc_pre;
-            float E[6];
+            float D[3], E[6], J[3];
 #pragma unroll
-            for (int k = 0; k < 6; ++k) E[k] = K * va_get<S>(s.E[k], a);
-            A.G[a][0] = add2(A.G[a][0], f2(E[0], E[1]));
-            A.G[a][1] = add2(A.G[a][1], f2(E[2], E[3]));
-            A.G[a][2] = add2(A.G[a][2], f2(E[4], E[5]));
-            if constexpr (HC)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) A.hf[a][k].x = fmaf(H, va_get<S>(s.D[k], a), A.hf[a][k].x);
-            if constexpr (!DRAG)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) A.hf[a][k].y = fmaf(K, va_get<S>(s.P[k], a), A.hf[a][k].y);
-            if (MODE == kSweep || a != b) {
-                const float w[3] = {ub[b][0] - c.u[a][0], ub[b][1] - c.u[a][1], ub[b][2] - c.u[a][2]};
-                A.hf[a][0].y = fmaf(E[0], w[0], fmaf(E[3], w[1], fmaf(E[4], w[2], A.hf[a][0].y)));
-                A.hf[a][1].y = fmaf(E[3], w[0], fmaf(E[1], w[1], fmaf(E[5], w[2], A.hf[a][1].y)));
-                A.hf[a][2].y = fmaf(E[4], w[0], fmaf(E[5], w[1], fmaf(E[2], w[2], A.hf[a][2].y)));
+            for (int k = 0; k < 3; ++k) {
+                D[k] = va_get<S>(s.D[k], a);
+                J[k] = va_get<S>(s.P[k], a);
+                E[k] = va_get<S>(s.E[k], a);
+                E[k + 3] = va_get<S>(s.E[k + 3], a);
             }
+            const float w[3] = {ub[b][0] - c.u[a][0], ub[b][1] - c.u[a][1], ub[b][2] - c.u[a][2]};
+            A.template add<DRAG, HC>(a, 0.5f * pr.vx_pre, -0.5f * pr.hc_pre, D, E, J, w, MODE == kSweep || a != b);
         }
     }
 }
@@ -347,7 +316,7 @@ __device__ __forceinline__ void pass1_cube(const mlbi_params &p, const float4 *s
 // is the previous sweep's (n - n_ref, u*) field, mom_c the moments, frest is
 // read, pst receives the sweep's u*)
 // the tile (bx, by, bz) of the tiled pass 1
-template <int S, int R, bool DRAG, int TY, int TX, int MODE>
+template <class T, int S, int R, bool DRAG, int MODE>
 __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *__restrict__ mom,
                                            const float *__restrict__ dg, const mlbi_entry *__restrict__ tab,
                                            const float4 *__restrict__ fext, const float4 *__restrict__ attr,
@@ -355,11 +324,11 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
                                            float4 *__restrict__ pst, int bx, int by, int bz)
 {
     constexpr bool HC = MODE == kExact;
-    using T = Tile<S, R, TY, TX>;
     extern __shared__ float4 smem[];
     float4 *sf = smem;                                                      // [NSLOT][S][PLANE]
     float *sg = reinterpret_cast<float *>(smem + (size_t)T::NSLOT * S * T::PLANE);   // [NSLOT][NP][PLANE]
-    const int x0 = bx * TX, y0 = by * TY, z0 = bz * p.zchunk;
+    float *red = reinterpret_cast<float *>(reinterpret_cast<char *>(smem) + T::ring) + T::sid();   // [SPLIT - 1][12 S][NT]
+    const int x0 = bx * T::TX, y0 = by * T::TY, z0 = bz * p.zchunk;
     const int z1 = min(z0 + p.zchunk, p.nz);
     const int x = x0 + T::lx(), y = y0 + T::ly();
     const bool active = x < p.nx && y < p.ny;
@@ -379,26 +348,34 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
             stage_plane<T, S>(p, xy, z + R + 1, ring(kz + R + 1, T::NSLOT), mom, dg, sf, sg);
             cp_async_commit();
         }
-        if (!active) continue;
+        if (T::SPLIT == 1 && !active) continue;
         const int cs = ring(kz, T::NSLOT);
         const long long r = x + (long long)p.nx * (y + (long long)p.ny * z);
-        float4 cv[S];
-#pragma unroll
-        for (int a = 0; a < S; ++a) cv[a] = sf[cs * S * T::PLANE + a * T::PLANE + cidx];
         Centre<S> c;
         float ub[S][3];
-        centre_of<S, MODE>(p, cv, mom_c, r, c, ub);
-        float dgc[T::NP];
-#pragma unroll
-        for (int q = 0; q < T::NP; ++q) dgc[q] = sg[cs * T::NP * T::PLANE + q * T::PLANE + cidx];
         Acc1<S> A;
         A.zero();
-        if constexpr (R == 1) {
-            pass1_cube<S, DRAG, MODE, T>(p, sf, sg, kz, cidx, c, ub, dgc, A);
-        } else {
-            PairW<S> w;
-            pair_weights<S>(p, dgc, w);
-            pass1_tile_shells<S, R, DRAG, TY, HC>(p, stab, sf, sg, kz, cidx, c, ub, w, A);
+        if (active) {
+            float4 cv[S];
+#pragma unroll
+            for (int a = 0; a < S; ++a) cv[a] = sf[cs * S * T::PLANE + a * T::PLANE + cidx];
+            centre_of<S, MODE>(p, cv, mom_c, r, c, ub);
+            if constexpr (R == 1) {
+                float dgc[T::NP];
+#pragma unroll
+                for (int q = 0; q < T::NP; ++q) dgc[q] = sg[cs * T::NP * T::PLANE + q * T::PLANE + cidx];
+                pass1_cube<S, DRAG, MODE, T>(p, sf, sg, kz, cidx, c, ub, dgc, A);
+            } else {
+                const TileView<S, T> view{sf, sg, kz, cidx, T::NSLOT};
+                p1_groups<S, T::SPLIT, DRAG, MODE == kSweep, HC>(p, stab, view, c.u, T::part(), A);
+            }
+        }
+        if constexpr (T::SPLIT > 1) {
+            if (active && T::part() > 0) A.put(red + (T::part() - 1) * 12 * S * T::NT, T::NT);
+            __syncthreads();
+            if (!active || T::part() > 0) continue;
+#pragma unroll
+            for (int k = 0; k < T::SPLIT - 1; ++k) A.take(red + k * 12 * S * T::NT, T::NT);
         }
         if constexpr (MODE == kSweep) {
             sweep_finish<S>(p, r, c, A, frest, pst);
@@ -422,24 +399,25 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
     }
 }
 
-// Resident blocks asked for: 4 leaves 128 registers a thread, enough for the
-// cube sums without spills (256^3 binary, reach 1: 0.867 ms; 5 blocks 0.892, 6
-// blocks 0.996, both spilling).  The loads from shared memory bound the kernel
-// (76 % of the L1's wavefronts at 128^3, issue slots 66 %).
-template <int S, int R, bool DRAG, int TY, int TX, int MODE>
-__global__ void __launch_bounds__(TX * TY, tile_blocks(Tile<S, R, TY, TX>::bytes, S <= 2 ? 4 : 2))
+// Resident blocks asked for: 16 warps at most, which leaves 128 registers a
+// thread, enough for the sums without spills (256^3 binary, reach 1: 4 blocks
+// 0.867 ms; 5 blocks 0.892, 6 blocks 0.996, both spilling).  The loads from
+// shared memory bound the kernel (76 % of the L1's wavefronts at 128^3, issue
+// slots 66 %).
+template <int S, int R, bool DRAG, int TX, int MODE>
+__global__ void __launch_bounds__(TileOf<S, R, TX>::NTH, TileOf<S, R, TX>::blocks)
     k_pass1_tiled(const mlbi_params p, const float4 *__restrict__ mom, const float *__restrict__ dg,
                   const mlbi_entry *__restrict__ tab, const float4 *__restrict__ fext, const float4 *__restrict__ attr,
                   const float4 *__restrict__ mom_c, float4 *__restrict__ frest, float4 *__restrict__ pst)
 {
     step_begin();
-    pass1_tile<S, R, DRAG, TY, TX, MODE>(p, mom, dg, tab, fext, attr, mom_c, frest, pst, blockIdx.x, blockIdx.y,
-                                     blockIdx.z);
+    pass1_tile<TileOf<S, R, TX>, S, R, DRAG, MODE>(p, mom, dg, tab, fext, attr, mom_c, frest, pst, blockIdx.x,
+                                                   blockIdx.y, blockIdx.z);
 }
 
 // every member of a group (block table entries {member, bx, by, bz}), the exact pass
-template <int S, int R, bool DRAG, int TY, int TX>
-__global__ void __launch_bounds__(TX * TY, tile_blocks(Tile<S, R, TY, TX>::bytes + sizeof(mlbi_params), S <= 2 ? 4 : 2))
+template <int S, int R, bool DRAG, int TX>
+__global__ void __launch_bounds__(TileOf<S, R, TX>::NTH, TileOf<S, R, TX>::blocks)
     k_pass1_group(const mlbi_member *__restrict__ mem, const int4 *__restrict__ blk)
 {
     __shared__ mlbi_params sp;
@@ -447,30 +425,83 @@ __global__ void __launch_bounds__(TX * TY, tile_blocks(Tile<S, R, TY, TX>::bytes
     const mlbi_member *m = mem + e.x;
     group_params(m, sp);
     const mlbi_buffers &b = m->b;
-    pass1_tile<S, R, DRAG, TY, TX, kExact>(sp, b.mom, b.dg, b.table, b.fext, b.attr, b.mom, b.frest, b.pst, e.y, e.z,
-                                       e.w);
+    pass1_tile<TileOf<S, R, TX>, S, R, DRAG, kExact>(sp, b.mom, b.dg, b.table, b.fext, b.attr, b.mom, b.frest, b.pst,
+                                                     e.y, e.z, e.w);
 }
 
 // launch the tiled pass 1 (or sweep: fld the previous sweep's field, out the next) of a lattice
-template <int S, int R, bool DRAG, int MODE, int TX = kBX>
+template <int S, int R, bool DRAG, int MODE, int TX = mlbi_tile_of(S, R).tx>
 cudaError_t launch_tiled(const mlbi_params &p, const mlbi_buffers &b, const float4 *fld, float4 *out, cudaStream_t s)
 {
-    constexpr int TY = TX == kBX ? mlbi_tile_ty(S, R) : 128 / TX;
-    if constexpr (TY == 0) {
+    if constexpr (mlbi_tile_ty(S, R) == 0) {
         return cudaErrorInvalidValue;
     } else {
         if constexpr (TX == kBX && R == 1 && S <= 2)
             if (p.tile_x == 16) return launch_tiled<S, R, DRAG, MODE, 16>(p, b, fld, out, s);
-        using T = Tile<S, R, TY, TX>;
-        auto k = k_pass1_tiled<S, R, DRAG, TY, TX, MODE>;
+        using T = TileOf<S, R, TX>;
+        auto k = k_pass1_tiled<S, R, DRAG, TX, MODE>;
         const size_t bytes = T::bytes + staged_table_bytes<T, R>(p);
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e != cudaSuccess) return e;
-        const dim3 g((unsigned)((p.nx + TX - 1) / TX), (unsigned)((p.ny + TY - 1) / TY),
+        const dim3 g((unsigned)((p.nx + T::TX - 1) / T::TX), (unsigned)((p.ny + T::TY - 1) / T::TY),
                      (unsigned)((p.nz + p.zchunk - 1) / p.zchunk));
-        return launch_step(k, g, dim3(kBX, T::NT / kBX), bytes, s, p, fld, b.dg, b.table, b.fext, b.attr, b.mom, b.frest,
+        return launch_step(k, g, dim3(kBX, T::NTH / kBX), bytes, s, p, fld, b.dg, b.table, b.fext, b.attr, b.mom, b.frest,
                            out);
     }
+}
+
+template <int S, int R, bool DRAG, int MODE = kExact>
+cudaError_t launch_pass1_tiled(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s)
+{
+    return launch_tiled<S, R, DRAG, MODE>(p, b, b.mom, b.pst, s);
+}
+
+template <int S, bool DRAG>
+cudaError_t launch_pass1(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s)
+{
+    if (p.hc_from_attr) {
+        // the surrogate's case only: binary, no drag-only mode, reach 1 or 2
+        if constexpr (S == 2 && !DRAG) {
+            if (p.tile_r == 1) return launch_pass1_tiled<S, 1, DRAG, kSurrogate>(p, b, s);
+            if (p.tile_r == 2) return launch_pass1_tiled<S, 2, DRAG, kSurrogate>(p, b, s);
+        }
+        return cudaErrorInvalidValue;
+    }
+    if (p.tile_r == 1) return launch_pass1_tiled<S, 1, DRAG>(p, b, s);
+    if (p.tile_r == 2) return launch_pass1_tiled<S, 2, DRAG>(p, b, s);
+    if (p.tile_r == 3) return launch_pass1_tiled<S, 3, DRAG>(p, b, s);
+    return launch_step(k_pass1<S, DRAG, kExact>, (unsigned)((p.N + 31) / 32), dim3(32, kParts), 0, s, p, b.mom, b.dg, b.table, b.fext,
+                       b.attr, b.mom, b.frest, b.pst);
+}
+
+template <int S>
+cudaError_t pass1_species(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s)
+{
+    return p.drag_only ? launch_pass1<S, true>(p, b, s) : launch_pass1<S, false>(p, b, s);
+}
+
+// ------------------------------------------------------------------ further sweeps (mlb_sweep*.cu)
+template <int S, int R, bool DRAG>
+cudaError_t launch_sweep_tiled(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next,
+                               cudaStream_t s)
+{
+    return launch_tiled<S, R, DRAG, kSweep>(p, b, prev, next, s);
+}
+
+template <int S, bool DRAG>
+cudaError_t launch_sweep(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next, cudaStream_t s)
+{
+    if (p.tile_r == 1) return launch_sweep_tiled<S, 1, DRAG>(p, b, prev, next, s);
+    if (p.tile_r == 2) return launch_sweep_tiled<S, 2, DRAG>(p, b, prev, next, s);
+    if (p.tile_r == 3) return launch_sweep_tiled<S, 3, DRAG>(p, b, prev, next, s);
+    return launch_step(k_pass1<S, DRAG, kSweep>, (unsigned)((p.N + 31) / 32), dim3(32, kParts), 0, s, p, prev, b.dg, b.table, b.fext,
+                       b.attr, b.mom, b.frest, next);
+}
+
+template <int S>
+cudaError_t sweep_species(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next, cudaStream_t s)
+{
+    return p.drag_only ? launch_sweep<S, true>(p, b, prev, next, s) : launch_sweep<S, false>(p, b, prev, next, s);
 }
 
 }  // namespace

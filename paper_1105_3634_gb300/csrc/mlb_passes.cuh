@@ -1,7 +1,6 @@
 // mlb_passes.cuh -- device code shared by the two force passes of a time step
-// (mlb_pass1.cu, mlb_pass2.cu): per-site pair weights, the arithmetic of one
-// +-d pair of a contact shell, the shared-memory z-marching tiles and the
-// compile-time offsets of the 3x3x3 cube.  Internal header.
+// (mlb_pass1.cuh, mlb_pass2.cuh): packed FP32 pairs, the shared-memory
+// z-marching tiles and the offset classes of the 3x3x3 cube.  Internal header.
 #pragma once
 
 #include "mlb_internal.h"
@@ -10,62 +9,6 @@
 #include <type_traits>
 
 namespace {
-
-// ------------------------------------------------------------------ pair weights
-// The midpoint contact value of Eqs. potmeanforce and gammaab between r and
-// r + d is (g(r) + g(r+d))/2 = B + dg(r+d)/2 with B = g_ref + dg(r)/2 and
-// dg = g - g_ref.  Per site and pair (a, b):
-//   exchange weight  vx_ab (g(r) + g(r+d))/2 = kp + k1 dg(r+d),  kp = vx_ab B,  k1 = vx_ab / 2
-//   hard core        -hc_ab [(g(r)+g(r+d))/2 n(r+d) - (g(r)+g(r-d))/2 n(r-d)]
-//                    = h (n(r+d) - n(r-d)) + c (n(r+d) dg(r+d) - n(r-d) dg(r-d)),
-//                    h = -hc_ab B,  c = -hc_ab / 2,
-// with n(r+d) - n(r-d) formed from the deviations n - n_ref (exact to rounding).
-template <int S>
-struct PairW {
-    static constexpr int NP = S * (S + 1) / 2;
-    float kp[NP], h[NP];
-};
-
-template <int S>
-__device__ __forceinline__ void pair_weights(const mlbi_params &p, const float *dgc, PairW<S> &w)
-{
-#pragma unroll
-    for (int q = 0; q < PairW<S>::NP; ++q) {
-        const float B = fmaf(0.5f, dgc[q], p.pair[q].g_ref);
-        w.kp[q] = p.pair[q].vx_pre * B;
-        w.h[q] = -p.pair[q].hc_pre * B;
-    }
-}
-
-// ------------------------------------------------------------------ one +-d pair of a shell
-// Pass 1 (inputs at r +- d: n, the n - n_ref difference dd, dg, and
-// jp/jm = s.(u^b(r +- d) - u^a(r))):
-//   t  = hard-core projection on s (Eq. potmeanforce),
-//   wn = h+ + h-, the friction weight, h+- = weight(r +- d) n^b(r +- d),
-//   sd = h+ jp + h- jm, the exchange projection (Eqs. gammaab, viscousforce);
-//   drag only: sd = -wn s.(u^a - u^b)(r), with sdu = s.(u^a - u^b).
-template <bool DRAG>
-__device__ __forceinline__ void pass1_point(float np, float nm, float dd, float jp, float jm, float dgp, float dgm,
-                                            float kp, float k1, float h, float c, float sdu, float &t, float &sd,
-                                            float &wn)
-{
-    const float gp = fmaf(k1, dgp, kp), gm = fmaf(k1, dgm, kp);
-    t = fmaf(h, dd, c * fmaf(np, dgp, -nm * dgm));
-    const float hp = gp * np, hm = gm * nm;
-    wn = hp + hm;
-    sd = DRAG ? -wn * sdu : fmaf(hp, jp, hm * jm);
-}
-
-// Pass 2: the same exchange projection at u*, jp/jm = s.(u*^b(r +- d) - u*^a(r))
-// (drag only: sdu = s.(u*^a - u*^b)(r)).
-template <bool DRAG>
-__device__ __forceinline__ float pass2_point(float np, float nm, float jp, float jm, float dgp, float dgm, float kp,
-                                             float k1, float sdu)
-{
-    const float gp = fmaf(k1, dgp, kp), gm = fmaf(k1, dgm, kp);
-    const float hp = gp * np, hm = gm * nm;
-    return DRAG ? -(hp + hm) * sdu : fmaf(hp, jp, hm * jm);
-}
 
 // ------------------------------------------------------------------ packed FP32 pairs
 // Pass 1 accumulates in lane pairs so that one packed instruction (two IEEE
@@ -77,44 +20,6 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 
-// accumulate one point with a unit vector s given at run time
-__device__ __forceinline__ void add_pass1(float sx, float sy, float sz, float t, float sd, float wn, float2 (&hf)[3],
-                                          float2 (&G)[3])
-{
-    const float2 tsd = f2(t, sd);
-    hf[0] = fma2(f2(sx, sx), tsd, hf[0]);
-    hf[1] = fma2(f2(sy, sy), tsd, hf[1]);
-    hf[2] = fma2(f2(sz, sz), tsd, hf[2]);
-    const float2 wxy = mul2(f2(wn, wn), f2(sx, sy));
-    const float wz = wn * sz;
-    G[0] = fma2(wxy, f2(sx, sy), G[0]);
-    G[1] = fma2(f2(wz, wxy.x), f2(sz, sy), G[1]);
-    G[2] = fma2(wxy, f2(sz, sz), G[2]);
-}
-
-// ------------------------------------------------------------------ neighbours from global memory
-// species-b data at r + sign d (n = 0 and u = 0 beyond a wall): n, the
-// deviation n - n_ref, the velocity, and the site index (-1 beyond a wall)
-struct Nb {
-    float dn, n, u0, u1, u2;
-    long long q;
-};
-
-template <bool INTERIOR>
-__device__ __forceinline__ Nb fetch_nb(const mlbi_params &p, const Loc &L, const float4 &e0, const float4 &e1,
-                                       int sign, const float4 *__restrict__ fld, float nref)
-{
-    Nb o;
-    o.q = INTERIOR ? L.r + sign * (long long)__float_as_int(e1.x) : nbr(p, L, e0, e1, sign);
-    if (INTERIOR || o.q >= 0) {
-        const float4 v = fld[o.q];
-        o.dn = v.x; o.n = nref + v.x; o.u0 = v.y; o.u1 = v.z; o.u2 = v.w;
-    } else {
-        o.dn = -nref; o.n = 0.f; o.u0 = 0.f; o.u1 = 0.f; o.u2 = 0.f;
-    }
-    return o;
-}
-
 // ------------------------------------------------------------------ shared-memory tiles (z marching)
 // A block of 32 x TY threads owns a 32 x TY column of sites and marches up z
 // through `zchunk` planes.  The stencil field of every species (float4: the
@@ -123,65 +28,52 @@ __device__ __forceinline__ Nb fetch_nb(const mlbi_params &p, const Loc &L, const
 // of (32 + 2R) x (TY + 2R) sites: 2R + 1 planes in use and one more being
 // filled by cp.async while the current plane is computed.  Every shell
 // neighbour is then read from shared memory.
-template <int S, int R, int TY_ = kBY, int TX_ = kBX>
+template <int S, int R, int TY_ = kBY, int TX_ = kBX, int SPLIT_ = 1>
 struct Tile {
-    static constexpr int TX = TX_, TY = TY_;
+    static constexpr int TX = TX_, TY = TY_, SPLIT = SPLIT_;
     static constexpr int TXH = TX + 2 * R, TYH = TY + 2 * R, PLANE = TXH * TYH;
     static constexpr int NSLOT = 2 * R + 2;
     static constexpr int NP = S * (S + 1) / 2;
-    static constexpr int NT = TX * TY;
-    static constexpr int J = (PLANE + NT - 1) / NT;          // staging sites per thread and plane
-    static constexpr size_t bytes = (size_t)NSLOT * PLANE * (S * sizeof(float4) + NP * sizeof(float));
-    static_assert(TX != kBX || bytes == (size_t)mlbi_tile_bytes(S, R, TY), "tile size formula");
-    // this thread's site of the tile
+    static constexpr int NT = TX * TY;                       // sites
+    static constexpr int NTH = NT * SPLIT;                   // threads: `split` per site, whole warps each
+    static_assert(NT % 32 == 0, "a warp has one part");
+    static constexpr int J = (PLANE + NTH - 1) / NTH;        // staging sites per thread and plane
+    static constexpr size_t ring = (size_t)NSLOT * PLANE * (S * sizeof(float4) + NP * sizeof(float));
+    static constexpr size_t bytes = ring + (size_t)(SPLIT - 1) * NT * 12 * S * sizeof(float);   // + partial sums
+    // resident blocks: what the tile's shared memory allows, 16 warps (128 registers) at most
+    static constexpr int by_smem = (int)((228 * 1024) / (bytes + 1024)), by_warps = NTH >= 512 ? 1 : 512 / NTH;
+    static constexpr int blocks = by_smem < 1 ? 1 : (by_smem < by_warps ? by_smem : by_warps);
+    // this thread's site of the tile, and its part of the site's shell sums
     static __device__ __forceinline__ int tid() { return threadIdx.y * kBX + threadIdx.x; }
-    static __device__ __forceinline__ int lx() { return TX == kBX ? threadIdx.x : tid() % TX; }
-    static __device__ __forceinline__ int ly() { return TX == kBX ? threadIdx.y : tid() / TX; }
+    static __device__ __forceinline__ int sid() { return SPLIT == 1 ? tid() : tid() % NT; }
+    static __device__ __forceinline__ int part() { return SPLIT == 1 ? 0 : tid() / NT; }
+    static __device__ __forceinline__ int lx() { return TX == kBX ? threadIdx.x : sid() % TX; }
+    static __device__ __forceinline__ int ly() { return TX == kBX && SPLIT == 1 ? threadIdx.y : sid() / TX; }
 };
 
-// The shell entries of the table-driven reach-3 tiles, staged once per block
-// into shared memory after the tile: the union shells' range of the table
-// where it fits (one block per SM holds the tile anyway), read there instead
-// of through the L1 on every shell point.  Host and device agree on the size.
-constexpr int kMaxStagedEntries = 512;
-__host__ __device__ inline int shell_entries(const mlbi_params &p, int &lo)
-{
-    lo = p.ushell_start[0];
-    int hi = lo;
-    for (int b = 0; b < p.S; ++b) {
-        lo = p.ushell_start[b] < lo ? p.ushell_start[b] : lo;
-        const int e = p.ushell_start[b] + p.ushell_count[b];
-        hi = e > hi ? e : hi;
-    }
-    return hi - lo;
-}
+// The tile of (S, R); reach 1 of one and two species also comes 16 x 8
+template <int S, int R, int TX>
+using TileOf = Tile<S, R, R == 1 ? 128 / TX : mlbi_tile_of(S, R).ty, TX, mlbi_tile_of(S, R).split>;
+
+// The shell groups of the reach-3 tiles, staged once per block into shared
+// memory after the tile where they fit (one block per SM holds the tile anyway),
+// read there instead of through the L1.  Host and device agree on the size.
 template <class T, int R>
 __host__ __device__ inline size_t staged_table_bytes(const mlbi_params &p)
 {
     if (R != 3) return 0;
-    int lo;
-    const int n = shell_entries(p, lo);
-    const size_t b = (size_t)n * 2 * sizeof(mlbi_entry);
-    return (n <= kMaxStagedEntries && T::bytes + b <= MLBI_MAX_TILE_BYTES) ? b : 0;
+    const size_t b = (size_t)p.grp[p.S - 1][7] * 2 * sizeof(mlbi_entry);
+    return T::bytes + b <= MLBI_MAX_TILE_BYTES ? b : 0;
 }
-// copy the entries to dst (visible after the caller's next barrier); returns
+// copy the groups to dst (visible after the caller's next barrier); returns
 // the table the shell loops read
 template <class T, int R>
 __device__ inline const mlbi_entry *stage_table(const mlbi_params &p, const mlbi_entry *tab, float4 *dst)
 {
+    tab += p.grp_at;
     if (staged_table_bytes<T, R>(p) == 0) return tab;
-    int lo;
-    const int n = shell_entries(p, lo);
-    const int nt = blockDim.x * blockDim.y, tid = threadIdx.y * blockDim.x + threadIdx.x;
-    for (int e = tid; e < 2 * n; e += nt) dst[e] = __ldg(&tab[2 * lo + e]);
-    return dst - 2 * lo;
-}
-
-// resident blocks per SM the tile's shared memory allows (at most `cap`)
-constexpr int tile_blocks(size_t bytes, int cap)
-{
-    const int b = (int)((228 * 1024) / (bytes + 1024));
-    return b < 1 ? 1 : (b > cap ? cap : b);
+    for (int e = T::tid(); e < 2 * p.grp[p.S - 1][7]; e += T::NTH) dst[e] = __ldg(&tab[e]);
+    return dst;
 }
 
 // (x, y) offsets x + nx y of this thread's staging sites, fixed while the
@@ -192,7 +84,7 @@ __device__ __forceinline__ void stage_sites(const mlbi_params &p, int x0, int y0
     const int tid = T::tid();
 #pragma unroll
     for (int j = 0; j < T::J; ++j) {
-        const int idx = tid + j * T::NT;
+        const int idx = tid + j * T::NTH;
         const int hx = idx % T::TXH, hy = idx / T::TXH;
         const int x = wrap_or_out(x0 - R + hx, p.nx, p.wall_axis == 0);
         const int y = wrap_or_out(y0 - R + hy, p.ny, p.wall_axis == 1);
@@ -221,7 +113,7 @@ __device__ __forceinline__ void stage_plane(const mlbi_params &p, const int (&xy
     const long long zoff = (long long)p.nx * p.ny * z;
 #pragma unroll
     for (int j = 0; j < T::J; ++j) {
-        const int idx = tid + j * T::NT;
+        const int idx = tid + j * T::NTH;
         if (j == T::J - 1 && idx >= T::PLANE) break;
         float4 *df = sf + (size_t)slot * S * T::PLANE + idx;
         float *dgs = sg + (size_t)slot * T::NP * T::PLANE + idx;

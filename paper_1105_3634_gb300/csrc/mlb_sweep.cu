@@ -4,34 +4,26 @@
 // velocity exchange F^v (Eqs. gammaab, viscousforce) now takes the partners'
 // velocities from the previous sweep's u*.  Pass 1 is the first sweep; each
 // further sweep is one more pass over the contact shells (device code in
-// mlb_pass1.cuh, mode kSweep).
+// mlb_pass1.cuh, mode kSweep).  One and two species here, the others in
+// mlb_sweep_s3.cu and mlb_sweep_s4.cu.
 #include "mlb_pass1.cuh"
 
-namespace {
-
-template <int S, int R, bool DRAG>
-cudaError_t launch_sweep_tiled(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next,
-                               cudaStream_t s)
+template <>
+cudaError_t mlbi_sweep_species<1>(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next,
+                                  cudaStream_t s)
 {
-    return launch_tiled<S, R, DRAG, kSweep>(p, b, prev, next, s);
+    return sweep_species<1>(p, b, prev, next, s);
 }
-
-template <int S, bool DRAG>
-cudaError_t launch_sweep(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next, cudaStream_t s)
+template <>
+cudaError_t mlbi_sweep_species<2>(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next,
+                                  cudaStream_t s)
 {
-    if (p.tile_r == 1) return launch_sweep_tiled<S, 1, DRAG>(p, b, prev, next, s);
-    if (p.tile_r == 2) return launch_sweep_tiled<S, 2, DRAG>(p, b, prev, next, s);
-    if (p.tile_r == 3) return launch_sweep_tiled<S, 3, DRAG>(p, b, prev, next, s);
-    return launch_step(k_pass1<S, DRAG, kSweep>, tiled_grid(p), dim3(kBX, kBY), 0, s, p, prev, b.dg, b.table, b.fext,
-                       b.attr, b.mom, b.frest, next);
+    return sweep_species<2>(p, b, prev, next, s);
 }
-
-}  // namespace
 
 cudaError_t mlbi_launch_sweep(const mlbi_params &p, const mlbi_buffers &b, const float4 *prev, float4 *next,
                               cudaStream_t s)
 {
-    if (p.drag_only) { MLBI_DISPATCH_S(return (launch_sweep<SS, true>(p, b, prev, next, s))); }
-    MLBI_DISPATCH_S(return (launch_sweep<SS, false>(p, b, prev, next, s)));
+    MLBI_DISPATCH_S(return mlbi_sweep_species<SS>(p, b, prev, next, s));
     return cudaErrorInvalidValue;
 }

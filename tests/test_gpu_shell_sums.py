@@ -122,3 +122,32 @@ def test_unaligned_rows(gpu, orc, name):
         out.append(sim.populations()[0])
         sim.close()
     assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
+
+
+# reach 2 and 3: shells from sign groups, one to three threads per site, tiles of 32 and 16
+GROUPS = {
+    "one_reach2": dict(sigma=[2.0], shape=(34, 5, 9)),
+    "one_reach3_drag": dict(sigma=[3.0], shape=(33, 9, 7), drag_only=True),
+    "two_reach2": dict(sigma=[1.5, 2.0], shape=(31, 6, 14), wall_axis=1),
+    "two_reach3": dict(sigma=[2.0, 3.0], shape=(35, 17, 6), wall_axis=2),
+    "two_reach3_drag": dict(sigma=[1.0, 3.0], shape=(8, 7, 20), drag_only=True),
+    "two_reach3_sweeps": dict(sigma=[2.0, 3.0], shape=(32, 8, 13), predictor_sweeps=3),
+    "three_reach2": dict(sigma=[1.0, 1.5, 2.0], shape=(33, 6, 7)),
+    "three_reach3": dict(sigma=[2.0, 2.5, 3.0], shape=(17, 9, 10), wall_axis=0),
+    "three_reach3_drag": dict(sigma=[1.0, 2.0, 3.0], shape=(16, 8, 7), drag_only=True),
+    "three_reach3_sweeps": dict(sigma=[2.0, 2.5, 3.0], shape=(31, 7, 8), predictor_sweeps=2, wall_axis=1),
+    "one_reach4": dict(sigma=[4.0], shape=(9, 7, 6)),
+    "two_reach8": dict(sigma=[8.0, 4.0], shape=(19, 11, 10), wall_axis=1),
+    "two_reach5_drag": dict(sigma=[5.0, 1.5], shape=(33, 8, 7), wall_axis=0, drag_only=True),
+    "two_reach4_sweeps": dict(sigma=[4.0, 3.0], shape=(11, 9, 13), wall_axis=2, predictor_sweeps=2),
+    "three_reach4": dict(sigma=[4.0, 2.0, 3.0], shape=(10, 9, 8)),
+    "four_reach3": dict(sigma=[1.5, 2.0, 2.5, 3.0], shape=(13, 9, 8), wall_axis=1),
+    "four_reach2": dict(sigma=[1.0, 1.5, 1.75, 2.0], shape=(33, 5, 6), wall_axis=2),
+}
+
+
+@pytest.mark.parametrize("name", sorted(GROUPS))
+def test_group_shells(gpu, orc, name):
+    lat = W.Lattice(**GROUPS[name])
+    n, u = fields(lat, 0.12)
+    check(gpu, orc, lat, n, u, 3)
