@@ -337,26 +337,61 @@ mlb_status rebuild(mlb_ctx *c)
         maxoff = std::max(maxoff, std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))));
     };
     auto count = [&]() { return (int)(tab.size() / 2); };
-    // an offset of a contact shell: the kernels read sign groups, the bounds on
+    // an offset of a contact shell or smoothing ball: the kernels read sign groups, the bounds on
     // offsets and on the shells' size hold for every offset
-    size_t shell_offsets = 0;
+    size_t shell_offsets = 0;           // shells and smoothing balls
     auto note = [&](int dx, int dy, int dz) {
         const long long lin = dx + nx * dy + nxy * dz;
         if (lin >= (1ll << 31) || lin <= -(1ll << 31)) lin_overflow = true;
         maxoff = std::max(maxoff, std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))));
         ++shell_offsets;
     };
-    // smoothing balls |d| <= kappa sigma_c (origin included)
+    // sign groups (mlb_groups.cuh) of the offsets that `mask` accepts (d != 0, up to R per
+    // axis), type by type; returns the end
+    auto push_groups = [&](int R, int first, int (&grp)[8], auto &&mask_of) {
+        int n = first;
+        for (int type = 0; type < 7; ++type) {
+            grp[type] = n;
+            // which of X, Y, Z are non-zero
+            const int has = type < 3 ? 1 << type : (type == 3 ? 3 : (type == 4 ? 5 : (type == 5 ? 6 : 7)));
+            for (int Z = (has & 4) ? 1 : 0; Z <= ((has & 4) ? R : 0); ++Z)
+                for (int Y = (has & 2) ? 1 : 0; Y <= ((has & 2) ? R : 0); ++Y)
+                    for (int X = (has & 1) ? 1 : 0; X <= ((has & 1) ? R : 0); ++X) {
+                        const int mask = mask_of(X, Y, Z);
+                        if (!mask) continue;
+                        const double len = std::sqrt((double)(X * X + Y * Y + Z * Z));
+                        mlbi_entry e0, e1;
+                        e0.x = (float)(X / len); e0.y = (float)(Y / len); e0.z = (float)(Z / len);
+                        std::memcpy(&e0.w, &mask, sizeof(int));
+                        std::memcpy(&e1.x, &X, sizeof(int));
+                        std::memcpy(&e1.y, &Y, sizeof(int));
+                        std::memcpy(&e1.z, &Z, sizeof(int));
+                        e1.w = 0.f;
+                        tab.push_back(e0);
+                        tab.push_back(e1);
+                        ++n;
+                    }
+        }
+        grp[7] = n;
+        return n;
+    };
+    // smoothing balls |d| <= kappa sigma_c; the kernel adds the site itself
+    int ball_count[MLBI_MAXS] = {0};
+    int nball = 0;
+    p.ball_at = (int)tab.size();
     for (int g = 0; g < S; ++g) {
-        double R = c->desc.kappa * c->sigma[g];
-        int Ri = (int)std::floor(R) + 1;
-        p.ball_start[g] = count();
+        const double R = c->desc.kappa * c->sigma[g];
+        const int Ri = (int)std::floor(R) + 1;
         for (int dz = -Ri; dz <= Ri; ++dz)
             for (int dy = -Ri; dy <= Ri; ++dy)
                 for (int dx = -Ri; dx <= Ri; ++dx)
-                    if ((double)(dx * dx + dy * dy + dz * dz) <= R * R) push(dx, dy, dz, 0, 0, 0, 0);
-        p.ball_count[g] = count() - p.ball_start[g];
-        p.ball_inv[g] = 1.0f / (float)p.ball_count[g];
+                    if ((double)(dx * dx + dy * dy + dz * dz) <= R * R) {
+                        note(dx, dy, dz);
+                        ++ball_count[g];
+                    }
+        nball = push_groups(Ri, nball, p.ball_grp[g],
+                            [&](int X, int Y, int Z) { return (double)(X * X + Y * Y + Z * Z) <= R * R ? 1 : 0; });
+        p.ball_inv[g] = 1.0f / (float)ball_count[g];
     }
     auto in_shell = [](double sab, int dx, int dy, int dz) {
         const double q = (double)(dx * dx + dy * dy + dz * dz), lo = sab - 0.5, hi = sab + 0.5;
@@ -419,32 +454,13 @@ mlb_status rebuild(mlb_ctx *c)
     for (int b = 0; b < S; ++b) {
         int R = 1;
         for (int a = 0; a < S; ++a) R = std::max(R, (int)std::ceil(0.5 * (c->sigma[a] + c->sigma[b]) + 0.5) + 1);
-        for (int type = 0; type < 7; ++type) {
-            p.grp[b][type] = ngroups;
-            // which of X, Y, Z are non-zero, as in mlb_groups.cuh
-            const int has = type < 3 ? 1 << type : (type == 3 ? 3 : (type == 4 ? 5 : (type == 5 ? 6 : 7)));
-            for (int Z = (has & 4) ? 1 : 0; Z <= ((has & 4) ? R : 0); ++Z)
-                for (int Y = (has & 2) ? 1 : 0; Y <= ((has & 2) ? R : 0); ++Y)
-                    for (int X = (has & 1) ? 1 : 0; X <= ((has & 1) ? R : 0); ++X) {
-                        int mask = 0;
-                        for (int a = 0; a < S; ++a)
-                            if (in_shell(0.5 * (c->sigma[a] + c->sigma[b]), X, Y, Z)) mask |= 1 << a;
-                        if (!mask) continue;
-                        shell_offsets += type < 3 ? 1 : (type < 6 ? 2 : 4);
-                        const double len = std::sqrt((double)(X * X + Y * Y + Z * Z));
-                        mlbi_entry e0, e1;
-                        e0.x = (float)(X / len); e0.y = (float)(Y / len); e0.z = (float)(Z / len);
-                        std::memcpy(&e0.w, &mask, sizeof(int));
-                        std::memcpy(&e1.x, &X, sizeof(int));
-                        std::memcpy(&e1.y, &Y, sizeof(int));
-                        std::memcpy(&e1.z, &Z, sizeof(int));
-                        e1.w = 0.f;
-                        tab.push_back(e0);
-                        tab.push_back(e1);
-                        ++ngroups;
-                    }
-        }
-        p.grp[b][7] = ngroups;
+        ngroups = push_groups(R, ngroups, p.grp[b], [&](int X, int Y, int Z) {
+            int mask = 0;
+            for (int a = 0; a < S; ++a)
+                if (in_shell(0.5 * (c->sigma[a] + c->sigma[b]), X, Y, Z)) mask |= 1 << a;
+            if (mask) shell_offsets += ((X != 0) + (Y != 0) + (Z != 0)) == 3 ? 4 : (((X != 0) + (Y != 0) + (Z != 0)) == 2 ? 2 : 1);
+            return mask;
+        });
     }
     if (attraction) maxoff = std::max(maxoff, attr_reach);
     // column form of the attraction: the region sigma_ab <= |d| <= lambda_c sigma_ab
@@ -507,7 +523,7 @@ mlb_status rebuild(mlb_ctx *c)
     if (lin_overflow) return fail(c, MLB_EINVAL, "stencil offsets exceed 32-bit linear offsets on this lattice");
     // the capacity counts every shell offset (two float4) as well as the tables;
     // the groups' entries, fewer than their offsets, are within it
-    const size_t need = tab.size() - 2 * (size_t)ngroups + 2 * shell_offsets;
+    const size_t need = tab.size() - 2 * (size_t)(ngroups + nball) + 2 * shell_offsets;
     if (need > 2 * (size_t)kTableCap)
         return fail(c, MLB_EINVAL, "stencil tables need %d float4, capacity is %d (reduce sigma or lambda_c)",
                     (int)need, 2 * kTableCap);
@@ -521,7 +537,7 @@ mlb_status rebuild(mlb_ctx *c)
     p.has_attraction = attraction ? 1 : 0;
     p.local_g = 1;
     for (int g = 0; g < S; ++g)
-        if (p.ball_count[g] != 1) p.local_g = 0;
+        if (ball_count[g] != 1) p.local_g = 0;
     p.tile_r = tile_r;
     p.attr_r = attraction ? attr_r : 0;
     p.tile_x = mlbi_tile_x(S, tile_r, c->desc.nx, c->desc.ny);

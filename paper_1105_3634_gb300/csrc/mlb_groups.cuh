@@ -265,14 +265,14 @@ __device__ __forceinline__ void p1_group(const Group &g, const V &v, float nr, c
     }
 }
 
-// the groups of neighbour species b that are `part` modulo PARTS in the table
+// the groups [grp[0], grp[7]) that are `part` modulo PARTS in the table, type by type
 // (so a type's odd one out falls to another part than the last type's)
 template <int PARTS, class F>
-__device__ __forceinline__ void for_groups(const mlbi_params &p, const float4 *tab, int b, int part, F &&f)
+__device__ __forceinline__ void for_groups(const int (&grp)[8], const float4 *tab, int part, F &&f)
 {
     static_for<0, 7>([&](auto TY) {
         constexpr int type = decltype(TY)::value;
-        const int start = p.grp[b][type], end = p.grp[b][type + 1];
+        const int start = grp[type], end = grp[type + 1];
         const int first = PARTS == 1 ? 0 : (part + PARTS - start % PARTS) % PARTS;
 #pragma unroll 1
         for (int k = start + first; k < end; k += PARTS) f(TY, Group(tab, k));
@@ -298,7 +298,7 @@ __device__ __forceinline__ void p1_groups(const mlbi_params &p, const float4 *ta
             for (int k = 0; k < 3; ++k) s.D[a][k] = s.P[a][k] = s.E[a][k] = s.E[a][k + 3] = 0.f;
         }
         const float nr = p.nref[b];
-        for_groups<PARTS>(p, tab, b, part, [&](auto TY, const Group &g) {
+        for_groups<PARTS>(p.grp[b], tab, part, [&](auto TY, const Group &g) {
             p1_group<S, b, DRAG, HC, decltype(TY)::value>(g, v, nr, Gc, ub, s);
         });
 #pragma unroll
@@ -374,7 +374,7 @@ __device__ __forceinline__ void p2_groups(const mlbi_params &p, const float4 *ta
             P[a][0] = P[a][1] = P[a][2] = 0.f;
         }
         const float nr = p.nref[b];
-        for_groups<PARTS>(p, tab, b, part, [&](auto TY, const Group &g) {
+        for_groups<PARTS>(p.grp[b], tab, part, [&](auto TY, const Group &g) {
             p2_group<S, b, DRAG, decltype(TY)::value>(g, v, nr, Gc, w, ub, P);
         });
 #pragma unroll

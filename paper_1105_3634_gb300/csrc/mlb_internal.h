@@ -51,7 +51,7 @@ struct mlbi_params {
     float xi2_coef[MLBI_MAXS];       // (pi/6) sigma^2
     float xi3_coef[MLBI_MAXS];       // (pi/6) sigma^3
     float xi2_ref, xi3_ref;
-    int ball_start[MLBI_MAXS], ball_count[MLBI_MAXS];
+    int ball_at, ball_grp[MLBI_MAXS][8];   // smoothing balls without their centre, as sign groups (see grp)
     float ball_inv[MLBI_MAXS];
     int reach;                       // largest offset component of any stencil (>= 1)
     int local_g;                     // every smoothing ball is the single site

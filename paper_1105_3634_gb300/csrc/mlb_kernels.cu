@@ -26,6 +26,7 @@
 #include "mlb_device.cuh"
 #include "mlb_collide.cuh"
 #include "mlb_popsum.cuh"
+#include "mlb_groups.cuh"
 
 #include <math.h>
 
@@ -110,31 +111,46 @@ __global__ void __launch_bounds__(kBlock) k_moments(const mlbi_params p, const f
 }
 
 // ------------------------------------------------------------------ contact values
-__global__ void __launch_bounds__(kBX * kBY) k_gfield(mlbi_params p, const float4 *__restrict__ mom,
-                                                      const mlbi_entry *__restrict__ tab, float *__restrict__ dg,
-                                                      unsigned int *__restrict__ flags)
+// The densities smoothed over the balls and the contact values of one site per
+// thread.  The balls are read as sign groups (mlb_groups.cuh): up to 8
+// independent loads, two wrapped coordinates per axis (sigma = 2 / 3, 128^3,
+// balls of 7 and 19 sites: 0.133 -> 0.067 ms; sigma = 8 / 4, 80 x 40 x 40, balls of 257 and 33: 0.166 -> 0.050; one table entry and one
+// wrapped neighbour per ball site before).
+template <int S>
+__global__ void __launch_bounds__(kBlock) k_gfield(const mlbi_params p, const float4 *__restrict__ mom,
+                                                   const mlbi_entry *__restrict__ tab, float *__restrict__ dg,
+                                                   unsigned int *__restrict__ flags)
 {
     step_begin();
-    Loc L;
-    if (!locate(p, L)) return;
-    const long long N = p.N, r = L.r;
+    const long long N = p.N, r = blockIdx.x * (long long)kBlock + threadIdx.x;
+    if (r >= N) return;
+    const int r32 = (int)r, x = r32 % p.nx, yz = r32 / p.nx, y = yz % p.ny, z = yz / p.ny;
+    const GlobalView<S> v{p, mom, nullptr, x, y, z};
     float d2 = 0.f, d3 = 0.f;
-    for (int c = 0; c < p.S; ++c) {
-        float sum = 0.f;
-        int outside = 0;
-        for (int k = 0; k < p.ball_count[c]; ++k) {
-            const int e = p.ball_start[c] + k;
-            const long long q = nbr(p, L, __ldg(&tab[2 * e]), __ldg(&tab[2 * e + 1]), 1);
-            if (q < 0) ++outside;
-            else sum += mom[c * N + q].x;
-        }
-        // smoothed density minus n_ref; sites beyond a wall hold no particles
-        const float dnbar = (sum - (float)outside * p.nref[c]) * p.ball_inv[c];
+#pragma unroll
+    for (int c = 0; c < S; ++c) {
+        const float *dn = reinterpret_cast<const float *>(mom + c * N);       // n - n_ref, every fourth float
+        float sum = dn[4 * r];
+        for_groups<1>(p.ball_grp[c], tab + p.ball_at, 0, [&](auto TY, const Group &g) {
+            constexpr int type = decltype(TY)::value;
+            Neighbour P[grp_pairs(type)], M[grp_pairs(type)];
+            v.template neighbours<type>(g, P, M);
+            float s = 0.f;
+#pragma unroll
+            for (int k = 0; k < grp_pairs(type); ++k) {
+                // sites beyond a wall hold no particles: n - n_ref = -n_ref
+                const float a = dn[4 * (long long)P[k].f], b = dn[4 * (long long)M[k].f];
+                s += (P[k].ok ? a : -p.nref[c]) + (M[k].ok ? b : -p.nref[c]);
+            }
+            sum += s;
+        });
+        const float dnbar = sum * p.ball_inv[c];
         d2 += p.xi2_coef[c] * dnbar;
         d3 += p.xi3_coef[c] * dnbar;
     }
     if (!(p.xi3_ref + d3 < 1.f)) atomicOr(flags, MLBI_FLAG_XI3);
-    for (int q = 0; q < p.npairs; ++q) dg[q * N + r] = bmcsl_dev(p.pair[q].h, p.xi2_ref, p.xi3_ref, d2, d3);
+#pragma unroll
+    for (int q = 0; q < S * (S + 1) / 2; ++q) dg[q * N + r] = bmcsl_dev(p.pair[q].h, p.xi2_ref, p.xi3_ref, d2, d3);
 }
 
 // ------------------------------------------------------------------ moments with local contact values
@@ -310,15 +326,6 @@ __global__ void __launch_bounds__(kFinalThreads) k_conservation_final(mlbi_param
 
 }  // namespace
 
-#define MLBI_DISPATCH_S(...)                                                                       \
-    switch (p.S) {                                                                                 \
-    case 1: { constexpr int SS = 1; __VA_ARGS__; } break;                                          \
-    case 2: { constexpr int SS = 2; __VA_ARGS__; } break;                                          \
-    case 3: { constexpr int SS = 3; __VA_ARGS__; } break;                                          \
-    case 4: { constexpr int SS = 4; __VA_ARGS__; } break;                                          \
-    default: return cudaErrorInvalidValue;                                                         \
-    }
-
 cudaError_t mlbi_launch_moments(const mlbi_params &p, const mlbi_buffers &b, int cur, cudaStream_t s, bool sums)
 {
     if (sums) {
@@ -337,7 +344,9 @@ cudaError_t mlbi_launch_moments(const mlbi_params &p, const mlbi_buffers &b, int
 
 cudaError_t mlbi_launch_gfield(const mlbi_params &p, const mlbi_buffers &b, cudaStream_t s)
 {
-    return launch_step(k_gfield, tiled_grid(p), dim3(kBX, kBY), 0, s, p, b.mom, b.table, b.dg, b.flags);
+    MLBI_DISPATCH_S(return launch_step(k_gfield<SS>, (unsigned)((p.N + kBlock - 1) / kBlock), kBlock, 0, s, p, b.mom,
+                                       b.table, b.dg, b.flags));
+    return cudaErrorInvalidValue;
 }
 
 namespace {
