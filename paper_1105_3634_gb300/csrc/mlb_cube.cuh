@@ -162,7 +162,7 @@ struct CubeView {
         for (int k = 0; k < 3; ++k) {
             const int s = ring(kz - 1 + k, nsl);
             f[k] = s * S * T::PLANE + cidx;
-            g[k] = s * T::NP * T::PLANE + cidx;
+            g[k] = s * T::NP * T::GPLANE + T::gidx();
         }
     }
     template <int X, int Y, int Z>
@@ -173,7 +173,7 @@ struct CubeView {
     template <int X, int Y, int Z>
     __device__ __forceinline__ VA<S> dg(int b) const
     {
-        return va_make<S>([&](int a) { return sg[g[1 + Z] + pair_of(a, b, S) * T::PLANE + X + T::TXH * Y]; });
+        return va_make<S>([&](int a) { return sg[g[1 + Z] + pair_of(a, b, S) * T::GPLANE + X + T::GP * Y]; });
     }
 };
 

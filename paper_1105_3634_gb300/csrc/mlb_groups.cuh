@@ -69,39 +69,44 @@ struct Neighbour {
 template <int S, class T>
 struct TileView {
     static constexpr bool kWalls = false;
+    __device__ __forceinline__ bool walls() const { return false; }
     const float4 *sf;
     const float *sg;
     int kz, cidx, nsl;
     __device__ __forceinline__ Neighbour centre() const
     {
         const int pl = ring(kz, nsl);
-        return {pl * S * T::PLANE + cidx, pl * T::NP * T::PLANE + cidx, true};
+        return {pl * S * T::PLANE + cidx, pl * T::NP * T::GPLANE + T::gidx(), true};
     }
     template <int TYPE>
     __device__ __forceinline__ void neighbours(const Group &g, Neighbour (&P)[grp_pairs(TYPE)],
                                                Neighbour (&M)[grp_pairs(TYPE)]) const
     {
         const int up = ring(kz + (grp_has(TYPE, 2) ? g.Z : 0), nsl), dn = grp_has(TYPE, 2) ? ring(kz - g.Z, nsl) : up;
-        const int oy = g.Y * T::TXH;
+        const int oy = g.Y * T::TXH, gy = g.Y * T::GP, gc = T::gidx();
         static_for<0, grp_pairs(TYPE)>([&](auto K) {
             constexpr int k = decltype(K)::value;
-            int o = 0;
-            if constexpr (grp_has(TYPE, 0)) o += grp_neg(TYPE, 0, k) ? -g.X : g.X;
-            if constexpr (grp_has(TYPE, 1)) o += grp_neg(TYPE, 1, k) ? -oy : oy;
-            P[k] = {up * S * T::PLANE + cidx + o, up * T::NP * T::PLANE + cidx + o, true};
-            M[k] = {dn * S * T::PLANE + cidx - o, dn * T::NP * T::PLANE + cidx - o, true};
+            int o = 0, og = 0;
+            if constexpr (grp_has(TYPE, 0)) o = og = grp_neg(TYPE, 0, k) ? -g.X : g.X;
+            if constexpr (grp_has(TYPE, 1)) {
+                o += grp_neg(TYPE, 1, k) ? -oy : oy;
+                og += grp_neg(TYPE, 1, k) ? -gy : gy;
+            }
+            P[k] = {up * S * T::PLANE + cidx + o, up * T::NP * T::GPLANE + gc + og, true};
+            M[k] = {dn * S * T::PLANE + cidx - o, dn * T::NP * T::GPLANE + gc - og, true};
         });
     }
     __device__ __forceinline__ float4 field(int b, int f) const { return sf[f + b * T::PLANE]; }
-    __device__ __forceinline__ float dg(int q, int g) const { return sg[g + q * T::PLANE]; }
+    __device__ __forceinline__ float dg(int q, int g) const { return sg[g + q * T::GPLANE]; }
 };
 
 // global memory, for shells beyond the tiles: the coordinates of a group's 8
-// neighbours are two per axis, so their wraps cost 6 selects a group instead of
-// 24, and every site takes the same path wherever it lies
+// neighbours are two per axis, so their wraps cost 6 minima a group instead of
+// 24 selects, and every site takes the same path wherever it lies
 template <int S>
 struct GlobalView {
     static constexpr bool kWalls = true;
+    __device__ __forceinline__ bool walls() const { return p.wall_axis >= 0; }
     const mlbi_params &p;
     const float4 *__restrict__ fld;
     const float *__restrict__ dgv;
@@ -111,43 +116,54 @@ struct GlobalView {
         const int r = x + p.nx * (y + p.ny * z);
         return {r, r, true};
     }
-    // c + d on an axis of extent L: wrapped, or (beyond a wall) any site and bad
-    static __device__ __forceinline__ int at(int c, int L, bool wall, bool &bad)
+    // c + d and c - d on a periodic axis of extent L (d < L): the smaller of the two
+    // candidates as unsigned numbers
+    static __device__ __forceinline__ int above(int c, int L) { return (int)min((unsigned)c, (unsigned)(c - L)); }
+    static __device__ __forceinline__ int below(int c, int L) { return (int)min((unsigned)c, (unsigned)(c + L)); }
+    // both, or on a wall axis (uniform) any site in the place of one beyond the wall
+    static __device__ __forceinline__ void pair_at(int c, int d, int L, bool wall, int &up, int &dn, bool &bad_up,
+                                                   bool &bad_dn)
     {
-        const bool lo = c < 0, hi = c >= L;
-        bad = wall && (lo || hi);
-        return lo ? c + L : (hi ? c - L : c);
+        if (wall) {
+            bad_up = c + d >= L;
+            bad_dn = c - d < 0;
+            up = min(c + d, L - 1);
+            dn = max(c - d, 0);
+        } else {
+            up = above(c + d, L);
+            dn = below(c - d, L);
+        }
     }
     template <int TYPE>
     __device__ __forceinline__ void neighbours(const Group &g, Neighbour (&P)[grp_pairs(TYPE)],
                                                Neighbour (&M)[grp_pairs(TYPE)]) const
     {
-        // [0] at +, [1] at -
-        int xs[2] = {x, x}, ys[2] = {y, y}, zs[2] = {z, z};
-        bool bx[2] = {false, false}, by[2] = {false, false}, bz[2] = {false, false};
-        if constexpr (grp_has(TYPE, 0)) {
-            xs[0] = at(x + g.X, p.nx, p.wall_axis == 0, bx[0]);
-            xs[1] = at(x - g.X, p.nx, p.wall_axis == 0, bx[1]);
-        }
-        if constexpr (grp_has(TYPE, 1)) {
-            ys[0] = at(y + g.Y, p.ny, p.wall_axis == 1, by[0]);
-            ys[1] = at(y - g.Y, p.ny, p.wall_axis == 1, by[1]);
-        }
-        if constexpr (grp_has(TYPE, 2)) {
-            zs[0] = at(z + g.Z, p.nz, p.wall_axis == 2, bz[0]);
-            zs[1] = at(z - g.Z, p.nz, p.wall_axis == 2, bz[1]);
-        }
+        int xp = x, xm = x, yp = y, ym = y, zp = z, zm = z;
+        bool bad_up = false, bad_dn = false;               // along the wall axis
+        if constexpr (grp_has(TYPE, 0)) pair_at(x, g.X, p.nx, p.wall_axis == 0, xp, xm, bad_up, bad_dn);
+        if constexpr (grp_has(TYPE, 1)) pair_at(y, g.Y, p.ny, p.wall_axis == 1, yp, ym, bad_up, bad_dn);
+        if constexpr (grp_has(TYPE, 2)) pair_at(z, g.Z, p.nz, p.wall_axis == 2, zp, zm, bad_up, bad_dn);
+        const int nxy = p.nx * p.ny;
+        const int ypr = yp * p.nx, ymr = ym * p.nx, zpr = zp * nxy, zmr = zm * nxy;
+        const bool w = p.wall_axis >= 0;
         static_for<0, grp_pairs(TYPE)>([&](auto K) {
             constexpr int k = decltype(K)::value;
             constexpr int ix = grp_neg(TYPE, 0, k), iy = grp_neg(TYPE, 1, k);
-            const int rp = xs[ix] + p.nx * (ys[iy] + p.ny * zs[0]), rm = xs[1 - ix] + p.nx * (ys[1 - iy] + p.ny * zs[1]);
-            const bool okp = !(bx[ix] || by[iy] || bz[0]), okm = !(bx[1 - ix] || by[1 - iy] || bz[1]);
-            P[k] = {okp ? rp : 0, okp ? rp : 0, okp};
-            M[k] = {okm ? rm : 0, okm ? rm : 0, okm};
+            bool okp = true, okm = true;
+            if (w) {
+                // whether pair k's + neighbour goes down the wall axis
+                const bool down = (ix && p.wall_axis == 0) || (iy && p.wall_axis == 1);
+                okp = !(down ? bad_dn : bad_up);
+                okm = !(down ? bad_up : bad_dn);
+            }
+            P[k].f = P[k].g = (ix ? xm : xp) + ((iy ? ymr : ypr) + zpr);
+            M[k].f = M[k].g = (ix ? xp : xm) + ((iy ? ypr : ymr) + zmr);
+            P[k].ok = okp;
+            M[k].ok = okm;
         });
     }
-    __device__ __forceinline__ float4 field(int b, int f) const { return fld[b * p.N + f]; }
-    __device__ __forceinline__ float dg(int q, int g) const { return dgv[q * p.N + g]; }
+    __device__ __forceinline__ float4 field(int b, int f) const { return (fld + b * p.N)[f]; }
+    __device__ __forceinline__ float dg(int q, int g) const { return (dgv + q * p.N)[g]; }
 };
 
 // ------------------------------------------------------------------ sums over a group
@@ -222,7 +238,7 @@ __device__ __forceinline__ void p1_group(const Group &g, const V &v, float nr, c
     static_for<0, NPR>([&](auto K) {
         constexpr int k = decltype(K)::value;
         float4 vp = v.field(b, P[k].f), vm = v.field(b, M[k].f);
-        if constexpr (V::kWalls) {
+        if (V::kWalls && v.walls()) {
             vp.x = P[k].ok ? vp.x : -nr;
             vm.x = M[k].ok ? vm.x : -nr;
         }
@@ -322,7 +338,7 @@ __device__ __forceinline__ void p2_group(const Group &g, const V &v, float nr, c
     static_for<0, NPR>([&](auto K) {
         constexpr int k = decltype(K)::value;
         float4 vp = v.field(b, P[k].f), vm = v.field(b, M[k].f);
-        if constexpr (V::kWalls) {
+        if (V::kWalls && v.walls()) {
             vp.x = P[k].ok ? vp.x : -nr;
             vm.x = M[k].ok ? vm.x : -nr;
         }

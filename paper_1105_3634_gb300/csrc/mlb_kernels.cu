@@ -114,8 +114,9 @@ __global__ void __launch_bounds__(kBlock) k_moments(const mlbi_params p, const f
 // The densities smoothed over the balls and the contact values of one site per
 // thread.  The balls are read as sign groups (mlb_groups.cuh): up to 8
 // independent loads, two wrapped coordinates per axis (sigma = 2 / 3, 128^3,
-// balls of 7 and 19 sites: 0.133 -> 0.067 ms; sigma = 8 / 4, 80 x 40 x 40, balls of 257 and 33: 0.166 -> 0.050; one table entry and one
-// wrapped neighbour per ball site before).
+// balls of 7 and 19 sites: 0.133 -> 0.051 ms; sigma = 8 / 4, 80 x 40 x 40, balls
+// of 257 and 33: 0.166 -> 0.032; one table entry and one wrapped neighbour per
+// ball site before).
 template <int S>
 __global__ void __launch_bounds__(kBlock) k_gfield(const mlbi_params p, const float4 *__restrict__ mom,
                                                    const mlbi_entry *__restrict__ tab, float *__restrict__ dg,

@@ -220,13 +220,14 @@ __device__ __forceinline__ void centre_of(const mlbi_params &p, const float4 (&c
 // share the groups: enough warps for small lattices of large spheres (80 x 40 x
 // 40 has 4000 site warps for 152 SMs), no idle lanes at ragged widths, and the
 // parts read neighbouring rows at the same time.  Measured (sigma = 8 / 4, 925
-// pairs a site, 80 x 40 x 40): pass 1 1.419 -> 0.496 ms, pass 2 1.043 ->
-// 0.437 (one thread per site, a table entry per pair, every neighbour of a site near a
-// face wrapped by itself: three quarters of the sites).
+// pairs a site, 80 x 40 x 40): pass 1 1.419 -> 0.429 ms, pass 2 1.043 ->
+// 0.348 (one thread per site, a table entry per pair, every neighbour of a site near a
+// face wrapped by itself: three quarters of the sites).  Two or eight threads a site: 0.53 and 0.53.
+// Five blocks per SM: the L1 latency counts more than a few spills (4 blocks 0.443).
 constexpr int kParts = 4;
 
 template <int S, bool DRAG, int MODE>
-__global__ void __launch_bounds__(32 * kParts, 4) k_pass1(const mlbi_params p, const float4 *__restrict__ mom,
+__global__ void __launch_bounds__(32 * kParts, 5) k_pass1(const mlbi_params p, const float4 *__restrict__ mom,
                                                           const float *__restrict__ dg,
                                                           const mlbi_entry *__restrict__ tab,
                                                           const float4 *__restrict__ fext,
@@ -326,13 +327,13 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
     constexpr bool HC = MODE == kExact;
     extern __shared__ float4 smem[];
     float4 *sf = smem;                                                      // [NSLOT][S][PLANE]
-    float *sg = reinterpret_cast<float *>(smem + (size_t)T::NSLOT * S * T::PLANE);   // [NSLOT][NP][PLANE]
+    float *sg = reinterpret_cast<float *>(smem + (size_t)T::NSLOT * S * T::PLANE);   // [NSLOT][NP][GPLANE]
     float *red = reinterpret_cast<float *>(reinterpret_cast<char *>(smem) + T::ring) + T::sid();   // [SPLIT - 1][12 S][NT]
     const int x0 = bx * T::TX, y0 = by * T::TY, z0 = bz * p.zchunk;
     const int z1 = min(z0 + p.zchunk, p.nz);
     const int x = x0 + T::lx(), y = y0 + T::ly();
     const bool active = x < p.nx && y < p.ny;
-    const int cidx = (T::ly() + R) * T::TXH + T::lx() + R;
+    const int cidx = T::cidx();
     const mlbi_entry *stab =
         stage_table<T, R>(p, tab, reinterpret_cast<float4 *>(reinterpret_cast<char *>(smem) + T::bytes));
     int xy[T::J];
@@ -363,7 +364,7 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
             if constexpr (R == 1) {
                 float dgc[T::NP];
 #pragma unroll
-                for (int q = 0; q < T::NP; ++q) dgc[q] = sg[cs * T::NP * T::PLANE + q * T::PLANE + cidx];
+                for (int q = 0; q < T::NP; ++q) dgc[q] = sg[(cs * T::NP + q) * T::GPLANE + T::gidx()];
                 pass1_cube<S, DRAG, MODE, T>(p, sf, sg, kz, cidx, c, ub, dgc, A);
             } else {
                 const TileView<S, T> view{sf, sg, kz, cidx, T::NSLOT};

@@ -51,7 +51,7 @@ __device__ __forceinline__ void add_rest(float (&acc)[3], const float4 fr)
 // from global memory: 32 sites a block, kParts threads per site (as k_pass1)
 constexpr int kParts2 = 4;
 template <int S, bool DRAG>
-__global__ void __launch_bounds__(32 * kParts2, 4) k_pass2(const mlbi_params p, const float *__restrict__ dg,
+__global__ void __launch_bounds__(32 * kParts2, 5) k_pass2(const mlbi_params p, const float *__restrict__ dg,
                                                            const mlbi_entry *__restrict__ tab,
                                                            const float4 *__restrict__ frest,
                                                            const float4 *__restrict__ pst, float4 *__restrict__ acc_f,
@@ -114,7 +114,7 @@ __device__ __forceinline__ void pass2_site(const mlbi_params &p, const mlbi_entr
         const int cs = ring(kz, NSL);
         float dgc[T::NP];
 #pragma unroll
-        for (int q = 0; q < T::NP; ++q) dgc[q] = sg[cs * T::NP * T::PLANE + q * T::PLANE + cidx];
+        for (int q = 0; q < T::NP; ++q) dgc[q] = sg[(cs * T::NP + q) * T::GPLANE + T::gidx()];
         float us[S][3];
 #pragma unroll
         for (int a = 0; a < S; ++a) {
@@ -131,7 +131,7 @@ __device__ __forceinline__ void pass2_site(const mlbi_params &p, const mlbi_entr
 // One thread per site where the fused kernel also serves the lattice: the two
 // agree bit for bit.
 template <int S, int R, int TX>
-using Tile2Of = Tile<S, R, TileOf<S, R, TX>::TY, TX, R == 2 && S <= 2 ? 1 : TileOf<S, R, TX>::SPLIT>;
+using Tile2Of = Tile<S, R, TileOf<S, R, TX>::TY, TX, R == 2 && S <= 2 ? 1 : TileOf<S, R, TX>::SPLIT, TX == 16>;
 
 template <int S, int R, bool DRAG, int TX>
 __global__ void __launch_bounds__(Tile2Of<S, R, TX>::NTH, Tile2Of<S, R, TX>::blocks)
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(Tile2Of<S, R, TX>::NTH, Tile2Of<S, R, TX>::blo
     const int z1 = min(z0 + p.zchunk, p.nz);
     const int x = x0 + T::lx(), y = y0 + T::ly();
     const bool active = x < p.nx && y < p.ny;
-    const int cidx = (T::ly() + R) * T::TXH + T::lx() + R;
+    const int cidx = T::cidx();
     const mlbi_entry *stab =
         stage_table<T, R>(p, tab, reinterpret_cast<float4 *>(reinterpret_cast<char *>(smem) + T::bytes));
     int xy[T::J];
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kBX * kBY, S <= 2 ? 3 : 2) k_pass2_collide(con
     const int x = x0 + T::lx(), y = y0 + T::ly();
     const int tid = T::tid();
     const bool active = x < p.nx && y < p.ny;
-    const int cidx = (T::ly() + R) * T::TXH + T::lx() + R;
+    const int cidx = T::cidx();
     const long long sxy = x + (long long)p.nx * y, nxy = (long long)p.nx * p.ny;
     int xy[T::J];
     stage_sites<T, R>(p, x0, y0, xy);
@@ -364,7 +364,7 @@ __device__ __forceinline__ void pass2_collide_tma_tile(const mlbi_params &p, con
     const int x = x0 + T::lx(), y = y0 + T::ly();
     const int tid = T::tid();
     const bool active = x < p.nx && y < p.ny;
-    const int cidx = (T::ly() + R) * T::TXH + T::lx() + R;
+    const int cidx = T::cidx();
     const int sxy = x + p.nx * y, nxy = p.nx * p.ny;
     auto issue = [&](int z) {
         mbar_expect_tx(bar, F::tx_bytes);

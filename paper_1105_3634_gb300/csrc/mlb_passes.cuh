@@ -28,17 +28,23 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 // of (32 + 2R) x (TY + 2R) sites: 2R + 1 planes in use and one more being
 // filled by cp.async while the current plane is computed.  Every shell
 // neighbour is then read from shared memory.
-template <int S, int R, int TY_ = kBY, int TX_ = kBX, int SPLIT_ = 1>
+// ALT (16-wide tiles): a warp's two rows of 16 sites are two apart and the rows
+// of the contact values 24 floats, so that their 4-byte loads meet in no bank
+// (rows one apart at a pitch of 18 or 22 share most of theirs): 256 x 16^3 0.247 ->
+// 0.242 ms per step, three species at reach 3 (512 x 64 x 64) pass 2 1.061 -> 1.049.
+template <int S, int R, int TY_ = kBY, int TX_ = kBX, int SPLIT_ = 1, bool ALT = false>
 struct Tile {
     static constexpr int TX = TX_, TY = TY_, SPLIT = SPLIT_;
     static constexpr int TXH = TX + 2 * R, TYH = TY + 2 * R, PLANE = TXH * TYH;
+    static_assert(!ALT || (TX == 16 && TXH <= 24 && TY % 4 == 0), "two rows per warp");
+    static constexpr int GP = ALT ? 24 : TXH, GPLANE = GP * TYH;      // rows and planes of the contact values
     static constexpr int NSLOT = 2 * R + 2;
     static constexpr int NP = S * (S + 1) / 2;
     static constexpr int NT = TX * TY;                       // sites
     static constexpr int NTH = NT * SPLIT;                   // threads: `split` per site, whole warps each
     static_assert(NT % 32 == 0, "a warp has one part");
     static constexpr int J = (PLANE + NTH - 1) / NTH;        // staging sites per thread and plane
-    static constexpr size_t ring = (size_t)NSLOT * PLANE * (S * sizeof(float4) + NP * sizeof(float));
+    static constexpr size_t ring = NSLOT * ((size_t)PLANE * S * sizeof(float4) + (size_t)GPLANE * NP * sizeof(float));
     static constexpr size_t bytes = ring + (size_t)(SPLIT - 1) * NT * 12 * S * sizeof(float);   // + partial sums
     // resident blocks: what the tile's shared memory allows, 16 warps (128 registers) at most
     static constexpr int by_smem = (int)((228 * 1024) / (bytes + 1024)), by_warps = NTH >= 512 ? 1 : 512 / NTH;
@@ -48,12 +54,20 @@ struct Tile {
     static __device__ __forceinline__ int sid() { return SPLIT == 1 ? tid() : tid() % NT; }
     static __device__ __forceinline__ int part() { return SPLIT == 1 ? 0 : tid() / NT; }
     static __device__ __forceinline__ int lx() { return TX == kBX ? threadIdx.x : sid() % TX; }
-    static __device__ __forceinline__ int ly() { return TX == kBX && SPLIT == 1 ? threadIdx.y : sid() / TX; }
+    static __device__ __forceinline__ int ly()
+    {
+        if (TX == kBX && SPLIT == 1) return threadIdx.y;
+        const int s = sid();
+        return ALT ? (s >> 6) * 4 + ((s >> 5) & 1) + ((s >> 4) & 1) * 2 : s / TX;
+    }
+    // the site in a staged plane of the fields and of the contact values
+    static __device__ __forceinline__ int cidx() { return (ly() + R) * TXH + lx() + R; }
+    static __device__ __forceinline__ int gidx() { return (ly() + R) * GP + lx() + R; }
 };
 
 // The tile of (S, R); reach 1 of one and two species also comes 16 x 8
 template <int S, int R, int TX>
-using TileOf = Tile<S, R, R == 1 ? 128 / TX : mlbi_tile_of(S, R).ty, TX, mlbi_tile_of(S, R).split>;
+using TileOf = Tile<S, R, R == 1 ? 128 / TX : mlbi_tile_of(S, R).ty, TX, mlbi_tile_of(S, R).split, TX == 16>;
 
 // The shell groups of the reach-3 tiles, staged once per block into shared
 // memory after the tile where they fit (one block per SM holds the tile anyway),
@@ -116,18 +130,18 @@ __device__ __forceinline__ void stage_plane(const mlbi_params &p, const int (&xy
         const int idx = tid + j * T::NTH;
         if (j == T::J - 1 && idx >= T::PLANE) break;
         float4 *df = sf + (size_t)slot * S * T::PLANE + idx;
-        float *dgs = sg + (size_t)slot * T::NP * T::PLANE + idx;
+        float *dgs = sg + (size_t)slot * T::NP * T::GPLANE + (T::GP == T::TXH ? idx : idx / T::TXH * T::GP + idx % T::TXH);
         if (xy[j] < 0 || z < 0) {
 #pragma unroll
             for (int b = 0; b < S; ++b) df[b * T::PLANE] = make_float4(-p.nref[b], 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int q = 0; q < T::NP; ++q) dgs[q * T::PLANE] = 0.f;
+            for (int q = 0; q < T::NP; ++q) dgs[q * T::GPLANE] = 0.f;
         } else {
             const long long g = zoff + xy[j];
 #pragma unroll
             for (int b = 0; b < S; ++b) cp_async16(df + b * T::PLANE, fld + b * N + g);
 #pragma unroll
-            for (int q = 0; q < T::NP; ++q) cp_async4(dgs + q * T::PLANE, dg + q * N + g);
+            for (int q = 0; q < T::NP; ++q) cp_async4(dgs + q * T::GPLANE, dg + q * N + g);
         }
     }
 }
