@@ -463,53 +463,52 @@ mlb_status rebuild(mlb_ctx *c)
         });
     }
     if (attraction) maxoff = std::max(maxoff, attr_reach);
-    // column form of the attraction: the region sigma_ab <= |d| <= lambda_c sigma_ab
-    // cut into columns (dx, dy) of the half plane; per column and pair the
-    // profile k(dz) = 6 eps sigma^6 / |d|^8 (zero off the region) and dz k(dz)
+    // column form of the attraction (mlb_attraction.cu): groups of columns that
+    // share the profile k(dz) = 6 eps sigma^6 / |d|^8 (zero off the region
+    // sigma_ab <= |d| <= lambda_c sigma_ab)
     p.acol_start = p.acol_count = p.aw_start = 0;
     if (attraction && attr_r) {
-        struct Col { int dx, dy, E; };
+        struct Col { int X, Y, E; };
         std::vector<Col> cols;
         auto rc_of = [&](int a, int b) { return c->lambda_c[a * S + b] * 0.5 * (c->sigma[a] + c->sigma[b]); };
-        for (int dy = 0; dy <= attr_r; ++dy)
-            for (int dx = -attr_r; dx <= attr_r; ++dx) {
-                if (dy == 0 && dx < 0) continue;                    // half plane, (0, 0) kept
+        for (int Y = 0; Y <= attr_r; ++Y)
+            for (int X = Y; X <= attr_r; ++X) {
                 int E = -1;
                 for (int a = 0; a < S; ++a)
                     for (int b = a; b < S; ++b) {
                         if (c->eps[a * S + b] == 0.0) continue;
                         const double rc = rc_of(a, b), sab = 0.5 * (c->sigma[a] + c->sigma[b]);
                         for (int dz = 0; dz <= attr_r; ++dz) {
-                            const double q = (double)(dx * dx + dy * dy + dz * dz);
+                            const double q = (double)(X * X + Y * Y + dz * dz);
                             if (q > 0.0 && q >= sab * sab && q <= rc * rc) E = std::max(E, dz);
                         }
                     }
-                if (E >= 0) cols.push_back({dx, dy, E});
+                if (E >= 0) cols.push_back({X, Y, E});
             }
+        // far columns first: the sums grow from the small weights to the large ones, which
+        // keeps their rounding errors small
+        std::stable_sort(cols.begin(), cols.end(),
+                         [](const Col &u, const Col &v) { return u.X * u.X + u.Y * u.Y > v.X * v.X + v.Y * v.Y; });
         p.acol_start = (int)tab.size();                            // float4 index
         for (const Col &k : cols) {
             mlbi_entry e;
-            std::memcpy(&e.x, &k.dx, sizeof(int));
-            std::memcpy(&e.y, &k.dy, sizeof(int));
+            std::memcpy(&e.x, &k.X, sizeof(int));
+            std::memcpy(&e.y, &k.Y, sizeof(int));
             std::memcpy(&e.z, &k.E, sizeof(int));
             e.w = 0.f;
             tab.push_back(e);
         }
         p.acol_count = (int)cols.size();
-        std::vector<float> w;                                       // (k, dz k) pairs
+        std::vector<float> w;                                       // k
         for (const Col &k : cols)
             for (int a = 0; a < S; ++a)
                 for (int b = a; b < S; ++b) {
                     const double e = c->eps[a * S + b], sab = 0.5 * (c->sigma[a] + c->sigma[b]);
                     const double rc = rc_of(a, b), s6 = std::pow(sab, 6.0);
                     for (int dz = 0; dz <= attr_r; ++dz) {
-                        const double q = (double)(k.dx * k.dx + k.dy * k.dy + dz * dz);
+                        const double q = (double)(k.X * k.X + k.Y * k.Y + dz * dz);
                         const bool in = e != 0.0 && q > 0.0 && q >= sab * sab && q <= rc * rc;
-                        const double kk = in ? 6.0 * e * s6 / (q * q * q * q) : 0.0;
-                        // the (0, 0) column pairs with itself: its +-dz sum counts each point twice
-                        const double half = (k.dx == 0 && k.dy == 0) ? 0.5 : 1.0;
-                        w.push_back((float)kk);
-                        w.push_back((float)(half * dz * kk));
+                        w.push_back(in ? (float)(6.0 * e * s6 / (q * q * q * q)) : 0.f);
                     }
                 }
         while (w.size() % 4) w.push_back(0.f);

@@ -62,10 +62,10 @@ struct mlbi_params {
     int grp_at, grp[MLBI_MAXS][8];
     int cube_mask[MLBI_MAXP];        // tile_r == 1: bit k set when half offset k of the 3x3x3 cube is in S_ab
     int attr_r;                      // reach of the attraction if the column attraction kernel serves it (1..8), else 0
-    // column form of the attraction (attr_r > 0): acol_count columns (dx, dy) of the
-    // half plane, one float4 each at table[acol_start] = (dx, dy, E, 0) as int bits,
-    // E the largest |dz| any pair reaches on the column; their weights are float2
-    // (k, dz k) per (column, pair, dz = 0..attr_r) at ((float2 *)(table + aw_start))
+    // column form of the attraction (attr_r > 0): acol_count groups of columns (+-X, +-Y),
+    // (+-Y, +-X), X >= Y >= 0, one float4 each at table[acol_start] = (X, Y, E, 0) as int
+    // bits, E the largest |dz| any pair reaches there; their weights k are floats per
+    // (group, pair, dz = 0..attr_r) at ((float *)(table + aw_start))
     int acol_start, acol_count, aw_start;
     int tile_x;                      // tile width of the reach-1 passes of one and two species: 32 (x 4) or 16 (x 8)
     int zchunk;                      // planes per block of the tiled kernels
