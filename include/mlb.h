@@ -239,12 +239,15 @@ const char *mlb_kernel_name(int32_t k);
 /* Work decomposition tuner (no counterpart in the paper; the physics is
  * unchanged: every site's arithmetic is the same under every candidate, so
  * results are bitwise identical whatever it picks).  Times `trials` force +
- * collision passes from the current state for each candidate number of z
- * planes per block of the stencil kernels (4, 8, 12, 16, 32, not above nz) and,
- * where both exist, the fused and the split pass-2 + collision launches, and
- * keeps the fastest.  The state is untouched: a trial reads f[cur] and writes
- * the other population buffer, and cur is not advanced.  Synchronises the
- * context's stream.  zchunk_out / fused_out (may be NULL) receive the choice.
+ * collision passes from the current state for the default number of z planes
+ * per block of the stencil kernels (which follows the lattice's size), for each
+ * candidate number (4, 8, 12, 16, 32, not above nz) and, where both exist, for
+ * the fused and the split pass-2 + collision launches, and keeps the fastest;
+ * the default stays unless a candidate is faster.  The state is untouched: a
+ * trial reads f[cur] and writes the other population buffer, and cur is not
+ * advanced.  Synchronises the context's stream.  zchunk_out (may be NULL)
+ * receives the fastest of the candidates, fused_out (may be NULL) whether the
+ * fused launch is kept.
  * Errors: MLB_EINVAL for trials < 1, MLB_ESTATE before fields are set. */
 mlb_status mlb_autotune(mlb_ctx *ctx, int32_t trials, int32_t *zchunk_out, int32_t *fused_out);
 

@@ -360,7 +360,8 @@ class Simulation:
 
     def autotune(self, trials: int = 3):
         """Pick the planes per block and the fused/split pass-2 launch by timing
-        (state and results unchanged); returns (zchunk, fused)."""
+        (state and results unchanged; the default decomposition stays unless a
+        candidate is faster); returns (fastest candidate zchunk, fused)."""
         z = ctypes.c_int32()
         fu = ctypes.c_int32()
         self._check(lib.mlb_autotune(self.ctx, trials, ctypes.byref(z), ctypes.byref(fu)))
