@@ -311,7 +311,6 @@ mlb_status rebuild(mlb_ctx *c)
             const double sab = 0.5 * (c->sigma[a] + c->sigma[b]);
             shell_reach = std::max(shell_reach, (int)std::floor(std::sqrt(std::pow(sab + 0.5, 2) - 1e-9)));
         }
-    const int tile_r = mlbi_tile_ty(S, shell_reach) ? shell_reach : 0;
     // reach of the attraction regions (column attraction kernel if <= 8)
     int attr_reach = 0;
     for (int a = 0; a < S; ++a)
@@ -320,6 +319,12 @@ mlb_status rebuild(mlb_ctx *c)
                 attr_reach = std::max(attr_reach,
                                       (int)std::floor(c->lambda_c[a * S + b] * 0.5 * (c->sigma[a] + c->sigma[b]) + 1e-9));
     const int attr_r = (attr_reach >= 1 && attr_reach <= 8) ? attr_reach : 0;
+    // Four species at reach 2: the 204 KB tile leaves 8 warps per SM, too few for an attraction
+    // summed offset by offset (reach 10, per step: 61 x 45 x 37 between walls 28.0 ms on tiles,
+    // 13.0 from global memory; 24 x 20 x 16 3.52 and 2.35).  The tiles of fewer species hold 12 to 16 warps and
+    // gain from them.
+    const bool few_warps = S == 4 && shell_reach == 2 && attr_reach > 8;
+    const int tile_r = mlbi_tile_ty(S, shell_reach) && !few_warps ? shell_reach : 0;
     auto push = [&](int dx, int dy, int dz, double vx, double vy, double vz, int mask) {
         mlbi_entry e0, e1;
         e0.x = (float)vx; e0.y = (float)vy; e0.z = (float)vz;

@@ -108,11 +108,12 @@ struct Acc1 {
 };
 
 // attraction sum_{+d} K_ab(d) (n^b(r+d) - n^b(r-d)) from global memory (G term
-// of Eq. potmeanforce, RPA), for reaches the column kernel does not serve
-template <int S, bool INTERIOR>
+// of Eq. potmeanforce, RPA), for reaches the column kernel does not serve: the
+// offsets that are `part` modulo PARTS
+template <int S, int PARTS, bool INTERIOR>
 __device__ __forceinline__ void pass1_attraction(const mlbi_params &p, const Loc &L,
                                                  const float4 *__restrict__ mom,
-                                                 const mlbi_entry *__restrict__ tab, float (&at)[S][3])
+                                                 const mlbi_entry *__restrict__ tab, int part, float (&at)[S][3])
 {
     const long long N = p.N;
 #pragma unroll
@@ -123,7 +124,7 @@ __device__ __forceinline__ void pass1_attraction(const mlbi_params &p, const Loc
             const float *nb = reinterpret_cast<const float *>(mom + b * N);
             float s0 = 0.f, s1 = 0.f, s2 = 0.f;
 #pragma unroll 4
-            for (int k = pr.attr_start; k < pr.attr_start + pr.attr_count; ++k) {
+            for (int k = pr.attr_start + part; k < pr.attr_start + pr.attr_count; k += PARTS) {
                 const float4 e0 = __ldg(&tab[2 * k]);
                 const float4 e1 = __ldg(&tab[2 * k + 1]);
                 float vp, vm;
@@ -143,6 +144,31 @@ __device__ __forceinline__ void pass1_attraction(const mlbi_params &p, const Loc
             at[a][0] += s0; at[a][1] += s1; at[a][2] += s2;
         }
     }
+}
+// Added to the site's hard-core force, so that the parts add up as their shell sums
+// do.  The half region has thousands of offsets for a pair of species and outweighs the
+// shells, so every thread of a site takes its share.  Per step (left to the first part
+// of a site -> shared; one thread per site in brackets): spheres of 4 with tails to 10
+// sites, 64^3, 8.98 -> 2.32 ms (2.78); three of 2 / 2.5 / 3 to 9 sites between walls, 61 x 45 x 37,
+// 23.7 -> 8.6 (9.0); two of 4 / 3, the same box, 8.85 -> 3.35 (5.3).
+template <int S, int PARTS>
+__device__ __forceinline__ void far_attraction(const mlbi_params &p, int x, int y, int z, long long r,
+                                               const float4 *__restrict__ mom, const mlbi_entry *__restrict__ tab,
+                                               int part, Acc1<S> &A)
+{
+    Loc L;
+    L.x = x; L.y = y; L.z = z; L.r = r;
+    const int R = p.reach;
+    L.interior = x >= R && x < p.nx - R && y >= R && y < p.ny - R && z >= R && z < p.nz - R;
+    float at[S][3];
+#pragma unroll
+    for (int a = 0; a < S; ++a) at[a][0] = at[a][1] = at[a][2] = 0.f;
+    if (L.interior) pass1_attraction<S, PARTS, true>(p, L, mom, tab, part, at);
+    else pass1_attraction<S, PARTS, false>(p, L, mom, tab, part, at);
+#pragma unroll
+    for (int a = 0; a < S; ++a)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) A.hf[a][k].x += at[a][k];
 }
 
 // Finish pass 1 at one site.  rest = F^hc + G + F_ext and the exchange at u
@@ -224,10 +250,12 @@ __device__ __forceinline__ void centre_of(const mlbi_params &p, const float4 (&c
 // 0.348 (one thread per site, a table entry per pair, every neighbour of a site near a
 // face wrapped by itself: three quarters of the sites).  Two or eight threads a site: 0.53 and 0.53.
 // Five blocks per SM: the L1 latency counts more than a few spills (4 blocks 0.443).
+// One species has the registers for eight (sigma = 4, 64^3, per step: 5 blocks 0.169 ms, 8 blocks
+// 0.164; with tails to 10 sites 2.81 and 2.32).
 constexpr int kParts = 4;
 
 template <int S, bool DRAG, int MODE>
-__global__ void __launch_bounds__(32 * kParts, 5) k_pass1(const mlbi_params p, const float4 *__restrict__ mom,
+__global__ void __launch_bounds__(32 * kParts, S == 1 ? 8 : 5) k_pass1(const mlbi_params p, const float4 *__restrict__ mom,
                                                           const float *__restrict__ dg,
                                                           const mlbi_entry *__restrict__ tab,
                                                           const float4 *__restrict__ fext,
@@ -240,11 +268,7 @@ __global__ void __launch_bounds__(32 * kParts, 5) k_pass1(const mlbi_params p, c
     const long long N = p.N, r = blockIdx.x * 32ll + threadIdx.x;
     const int part = threadIdx.y;
     const bool active = r < N;
-    Loc L;
-    L.r = r;
-    L.x = (int)(r % p.nx);
-    L.y = (int)(r / p.nx % p.ny);
-    L.z = (int)(r / ((long long)p.nx * p.ny));
+    const int x = (int)(r % p.nx), y = (int)(r / p.nx % p.ny), z = (int)(r / ((long long)p.nx * p.ny));
     Centre<S> c;
     Acc1<S> A;
     A.zero();
@@ -254,8 +278,10 @@ __global__ void __launch_bounds__(32 * kParts, 5) k_pass1(const mlbi_params p, c
 #pragma unroll
         for (int a = 0; a < S; ++a) cv[a] = mom[a * N + r];
         centre_of<S, MODE>(p, cv, mom_c, r, c, ub);
-        const GlobalView<S> view{p, mom, dg, L.x, L.y, L.z};
+        const GlobalView<S> view{p, mom, dg, x, y, z};
         p1_groups<S, kParts, DRAG, MODE == kSweep, MODE == kExact>(p, tab + p.grp_at, view, c.u, part, A);
+        if constexpr (MODE == kExact)
+            if (p.has_attraction && !p.attr_r) far_attraction<S, kParts>(p, x, y, z, r, mom, tab, part, A);
         if (part > 0) A.put(&red[part - 1][0][threadIdx.x], 32);
     }
     __syncthreads();
@@ -272,11 +298,6 @@ __global__ void __launch_bounds__(32 * kParts, 5) k_pass1(const mlbi_params p, c
             const float4 v = attr[a * N + r];
             A.at[a][0] = v.x; A.at[a][1] = v.y; A.at[a][2] = v.z;
         }
-    } else if (p.has_attraction) {
-        const int R = p.reach;
-        L.interior = L.x >= R && L.x < p.nx - R && L.y >= R && L.y < p.ny - R && L.z >= R && L.z < p.nz - R;
-        if (L.interior) pass1_attraction<S, true>(p, L, mom, tab, A.at);
-        else pass1_attraction<S, false>(p, L, mom, tab, A.at);
     }
     pass1_finish<S, DRAG>(p, r, c, A, fext, frest, pst);
 }
@@ -370,6 +391,8 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
                 const TileView<S, T> view{sf, sg, kz, cidx, T::NSLOT};
                 p1_groups<S, T::SPLIT, DRAG, MODE == kSweep, HC>(p, stab, view, c.u, T::part(), A);
             }
+            if constexpr (MODE == kExact)
+                if (p.has_attraction && !p.attr_r) far_attraction<S, T::SPLIT>(p, x, y, z, r, mom, tab, T::part(), A);
         }
         if constexpr (T::SPLIT > 1) {
             if (active && T::part() > 0) A.put(red + (T::part() - 1) * 12 * S * T::NT, T::NT);
@@ -388,13 +411,6 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
                 const float4 v = attr[a * p.N + r];
                 A.at[a][0] = v.x; A.at[a][1] = v.y; A.at[a][2] = v.z;
             }
-        } else if (p.has_attraction) {
-            Loc L;
-            L.x = x; L.y = y; L.z = z; L.r = r;
-            const int Rr = p.reach;
-            L.interior = x >= Rr && x < p.nx - Rr && y >= Rr && y < p.ny - Rr && z >= Rr && z < p.nz - Rr;
-            if (L.interior) pass1_attraction<S, true>(p, L, mom, tab, A.at);
-            else pass1_attraction<S, false>(p, L, mom, tab, A.at);
         }
         pass1_finish<S, DRAG>(p, r, c, A, fext, frest, pst);
     }
