@@ -17,9 +17,17 @@
 // per dz and species before).
 // Each thread owns Z consecutive planes of one (x, y) site and streams the
 // planes: a plane's A and B are formed once and added to all Z outputs and both
-// output species (packed FP32x2), C is kept for the differences.  A block stages the deviations of
+// output species (packed FP32x2), C is kept for the differences.  A group's sums
+// are formed by themselves and added to the running ones once: with every plane added
+// straight in, several hundred terms, the error against 64 bits grew beyond that of a
+// sum by columns on many fields (sigma = 2 / 3, 40 x 20 x 18, largest error over
+// largest |G|, by half-plane columns / planes added straight in / this form:
+// wave along x 4.1e-7 / 9.0e-7 / 2.2e-7, along z 1.2e-6 / 2.3e-7 / 1.1e-7, noise 8.1e-7 /
+// 5.7e-7 / 2.6e-7).  An output's partial sum is live from its first plane to its last
+// only, which keeps two species within 128 registers.  A block stages the deviations of
 // one neighbour species over its (32 + 2R) x (TY + 2R) x (Z + 2R) slab in shared
-// memory.  (sigma = 2 / 3, reach 7, 128^3: 0.867 -> 0.707 ms.)
+// memory.  (sigma = 2 / 3, reach 7, 128^3: half-plane columns 0.868 ms, planes added
+// straight in 0.707, this form 0.742.)
 #include "mlb_internal.h"
 #include "mlb_device.cuh"
 #include "mlb_cube.cuh"
@@ -98,51 +106,62 @@ __global__ void __launch_bounds__(kBX * TY, 2) k_attraction_columns(const mlbi_p
                 // Opposite columns are subtracted first (what they share is exact to
                 // cancel), then C's planes z + dz and z - dz below.
                 float C[W];
+                VA<AG> t[Z][2];                              // this group's share of G_x, G_y
 #pragma unroll
                 for (int j = 0; j < W; ++j) {
                     C[j] = 0.f;
-                    if (j < R - E || j >= R + Z + E) continue;      // uniform: no output reaches this plane
-                    const float *v = centre + j * T::PL;
-                    float A, B;
-                    if (Y > 0 && X > Y) {
-                        const float pp = v[X + yr], pm = v[X - yr], mp = v[-X + yr], mm = v[-X - yr];
-                        const float qp = v[Y + xr], qm = v[Y - xr], rp = v[-Y + xr], rm = v[-Y - xr];
-                        const float d1 = pp - mm, d2 = pm - mp, e1 = qp - rm, e2 = qm - rp;
-                        A = fmaf(fx, d1 + d2, fy * (e1 + e2));
-                        B = fmaf(fy, d1 - d2, fx * (e1 - e2));
-                        C[j] = ((pp + mm) + (pm + mp)) + ((qp + rm) + (qm + rp));
-                    } else if (Y > 0) {
-                        const float pp = v[X + yr], pm = v[X - yr], mp = v[-X + yr], mm = v[-X - yr];
-                        const float d1 = pp - mm, d2 = pm - mp;
-                        A = fx * (d1 + d2);
-                        B = fx * (d1 - d2);
-                        C[j] = (pp + mm) + (pm + mp);
-                    } else if (X > 0) {
-                        const float xp = v[X], xm = v[-X], yp = v[xr], ym = v[-xr];
-                        A = fx * (xp - xm);
-                        B = fx * (yp - ym);
-                        C[j] = (xp + xm) + (yp + ym);
-                    } else {
-                        A = B = 0.f;
-                        C[j] = v[0];
-                    }
+                    if (j < Z) t[j][0] = t[j][1] = va_zero<AG>();
+                    if (j >= R - E && j < R + Z + E) {              // uniform: some output reaches this plane
+                        const float *v = centre + j * T::PL;
+                        float A, B;
+                        if (Y > 0 && X > Y) {
+                            const float pp = v[X + yr], pm = v[X - yr], mp = v[-X + yr], mm = v[-X - yr];
+                            const float qp = v[Y + xr], qm = v[Y - xr], rp = v[-Y + xr], rm = v[-Y - xr];
+                            const float d1 = pp - mm, d2 = pm - mp, e1 = qp - rm, e2 = qm - rp;
+                            A = fmaf(fx, d1 + d2, fy * (e1 + e2));
+                            B = fmaf(fy, d1 - d2, fx * (e1 - e2));
+                            C[j] = ((pp + mm) + (pm + mp)) + ((qp + rm) + (qm + rp));
+                        } else if (Y > 0) {
+                            const float pp = v[X + yr], pm = v[X - yr], mp = v[-X + yr], mm = v[-X - yr];
+                            const float d1 = pp - mm, d2 = pm - mp;
+                            A = fx * (d1 + d2);
+                            B = fx * (d1 - d2);
+                            C[j] = (pp + mm) + (pm + mp);
+                        } else if (X > 0) {
+                            const float xp = v[X], xm = v[-X], yp = v[xr], ym = v[-xr];
+                            A = fx * (xp - xm);
+                            B = fx * (yp - ym);
+                            C[j] = (xp + xm) + (yp + ym);
+                        } else {
+                            A = B = 0.f;
+                            C[j] = v[0];
+                        }
 #pragma unroll
-                    for (int i = 0; i < Z; ++i) {
-                        const int dz = j - R - i;
-                        if (dz < -R || dz > R) continue;
-                        const int m = dz < 0 ? -dz : dz;
-                        acc[i][0] = va_fma(A, k[m], acc[i][0]);
-                        acc[i][1] = va_fma(B, k[m], acc[i][1]);
+                        for (int i = 0; i < Z; ++i) {
+                            const int dz = j - R - i;
+                            if (dz < -R || dz > R) continue;
+                            const int m = dz < 0 ? -dz : dz;
+                            t[i][0] = va_fma(A, k[m], t[i][0]);
+                            t[i][1] = va_fma(B, k[m], t[i][1]);
+                        }
+                    }
+                    if (j >= 2 * R) {                               // output j - 2R has all its planes
+                        acc[j - 2 * R][0] = acc[j - 2 * R][0] + t[j - 2 * R][0];
+                        acc[j - 2 * R][1] = acc[j - 2 * R][1] + t[j - 2 * R][1];
                     }
                 }
+                VA<AG> tz[Z];
+#pragma unroll
+                for (int i = 0; i < Z; ++i) tz[i] = va_zero<AG>();
 #pragma unroll
                 for (int dz = 1; dz <= R; ++dz) {
                     if (dz > E) break;
                     const VA<AG> kz = (float)dz * k[dz];
 #pragma unroll
-                    for (int i = 0; i < Z; ++i)
-                        acc[i][2] = va_fma(C[i + R + dz] - C[i + R - dz], kz, acc[i][2]);
+                    for (int i = 0; i < Z; ++i) tz[i] = va_fma(C[i + R + dz] - C[i + R - dz], kz, tz[i]);
                 }
+#pragma unroll
+                for (int i = 0; i < Z; ++i) acc[i][2] = acc[i][2] + tz[i];
             }
         }
         if (x < p.nx && y < p.ny) {
