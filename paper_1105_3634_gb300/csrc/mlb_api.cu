@@ -472,6 +472,7 @@ mlb_status rebuild(mlb_ctx *c)
     // share the profile k(dz) = 6 eps sigma^6 / |d|^8 (zero off the region
     // sigma_ab <= |d| <= lambda_c sigma_ab)
     p.acol_start = p.acol_count = p.aw_start = 0;
+    size_t half_columns = 0, attr_entries = 0;
     if (attraction && attr_r) {
         struct Col { int X, Y, E; };
         std::vector<Col> cols;
@@ -488,7 +489,10 @@ mlb_status rebuild(mlb_ctx *c)
                             if (q > 0.0 && q >= sab * sab && q <= rc * rc) E = std::max(E, dz);
                         }
                     }
-                if (E >= 0) cols.push_back({X, Y, E});
+                if (E >= 0) {
+                    cols.push_back({X, Y, E});
+                    half_columns += X == 0 ? 1 : (Y == 0 || X == Y ? 2 : 4);
+                }
             }
         // far columns first: the sums grow from the small weights to the large ones, which
         // keeps their rounding errors small
@@ -523,11 +527,14 @@ mlb_status rebuild(mlb_ctx *c)
             e.x = w[i]; e.y = w[i + 1]; e.z = w[i + 2]; e.w = w[i + 3];
             tab.push_back(e);
         }
+        attr_entries = tab.size() - (size_t)p.acol_start;
     }
     if (lin_overflow) return fail(c, MLB_EINVAL, "stencil offsets exceed 32-bit linear offsets on this lattice");
-    // the capacity counts every shell offset (two float4) as well as the tables;
-    // the groups' entries, fewer than their offsets, are within it
-    const size_t need = tab.size() - 2 * (size_t)(ngroups + nball) + 2 * shell_offsets;
+    // the capacity counts every shell offset (two float4) and every column of the
+    // attraction's half plane with its (k, dz k) weights; the entries of the groups
+    // that stand for them, fewer, are within it
+    const size_t need = tab.size() - 2 * (size_t)(ngroups + nball) + 2 * shell_offsets - attr_entries + half_columns +
+                        (half_columns * (size_t)(np * (attr_r + 1) * 2) + 3) / 4;
     if (need > 2 * (size_t)kTableCap)
         return fail(c, MLB_EINVAL, "stencil tables need %d float4, capacity is %d (reduce sigma or lambda_c)",
                     (int)need, 2 * kTableCap);
