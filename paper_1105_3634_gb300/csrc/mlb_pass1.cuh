@@ -40,7 +40,7 @@ __device__ __forceinline__ void solve_sym3(const float G[6], const float b[3], f
 }
 
 // per species: hf[q] = (F^hc_q, F^v_q), G = friction matrix packed as
-// (xx, yy), (zz, xy), (xz, yz) (see add_pass1), at = attraction
+// (xx, yy), (zz, xy), (xz, yz), at = attraction
 template <int S>
 struct Acc1 {
     float2 hf[S][3], G[S][3];
@@ -249,13 +249,24 @@ __device__ __forceinline__ void centre_of(const mlbi_params &p, const float4 (&c
 // pairs a site, 80 x 40 x 40): pass 1 1.419 -> 0.429 ms, pass 2 1.043 ->
 // 0.348 (one thread per site, a table entry per pair, every neighbour of a site near a
 // face wrapped by itself: three quarters of the sites).  Two or eight threads a site: 0.53 and 0.53.
-// Five blocks per SM: the L1 latency counts more than a few spills (4 blocks 0.443).
-// One species has the registers for eight (sigma = 4, 64^3, per step: 5 blocks 0.169 ms, 8 blocks
-// 0.164; with tails to 10 sites 2.81 and 2.32).
+// Blocks per SM: two species take five, the L1 latency counts more than a few spills
+// (4 blocks 0.443).  Three and four species would spill 1.0 and 2.9 KB at five (per step, 64^3,
+// sigma = 6 / 4 / 3: 5 blocks 2.40 ms, 4 blocks 2.00, 3 blocks 2.08; 6 / 4 / 3 / 2: 5 blocks 8.6, 4 blocks
+// 3.13, 3 blocks 3.04, 2 blocks 3.80; one thread per site 6.08 and 9.40); drag-only sums need
+// fewer registers (four species of 1.5 / 2 / 2.5 / 3: 5 or 4 blocks 0.90 and 0.91, 3 blocks 0.975).  One species has the
+// registers for seven (sigma = 4: 5 blocks 0.170, 7 blocks 0.164, 8 blocks 0.169).
+// FAR: with an attraction beyond the columns' reach, whose loop wants warps more than
+// registers (four species of 4 / 2 / 3 / 3.5 to 10 sites between walls, 61 x 45 x 37: 5 blocks 13.2
+// ms, 3 blocks 16.7; one of 4 to 10 sites, 64^3: 5 blocks 2.81, 8 blocks 2.32), as a kernel of its own.
 constexpr int kParts = 4;
 
-template <int S, bool DRAG, int MODE>
-__global__ void __launch_bounds__(32 * kParts, S == 1 ? 8 : 5) k_pass1(const mlbi_params p, const float4 *__restrict__ mom,
+constexpr int pass1_blocks(int S, bool drag, bool far)
+{
+    return S == 1 ? (far ? 8 : 7) : S == 2 || far ? 5 : drag ? (S == 4 ? 4 : 5) : (S == 3 ? 4 : 3);
+}
+
+template <int S, bool DRAG, int MODE, bool FAR>
+__global__ void __launch_bounds__(32 * kParts, pass1_blocks(S, DRAG, FAR)) k_pass1(const mlbi_params p, const float4 *__restrict__ mom,
                                                           const float *__restrict__ dg,
                                                           const mlbi_entry *__restrict__ tab,
                                                           const float4 *__restrict__ fext,
@@ -280,8 +291,7 @@ __global__ void __launch_bounds__(32 * kParts, S == 1 ? 8 : 5) k_pass1(const mlb
         centre_of<S, MODE>(p, cv, mom_c, r, c, ub);
         const GlobalView<S> view{p, mom, dg, x, y, z};
         p1_groups<S, kParts, DRAG, MODE == kSweep, MODE == kExact>(p, tab + p.grp_at, view, c.u, part, A);
-        if constexpr (MODE == kExact)
-            if (p.has_attraction && !p.attr_r) far_attraction<S, kParts>(p, x, y, z, r, mom, tab, part, A);
+        if constexpr (FAR) far_attraction<S, kParts>(p, x, y, z, r, mom, tab, part, A);
         if (part > 0) A.put(&red[part - 1][0][threadIdx.x], 32);
     }
     __syncthreads();
@@ -418,7 +428,8 @@ __device__ __forceinline__ void pass1_tile(const mlbi_params &p, const float4 *_
 
 // Resident blocks asked for: 16 warps at most, which leaves 128 registers a
 // thread, enough for the sums without spills (256^3 binary, reach 1: 4 blocks
-// 0.867 ms; 5 blocks 0.892, 6 blocks 0.996, both spilling).  The loads from
+// 0.867 ms; 5 blocks 0.892, 6 blocks 0.996, both spilling).  The grouped kernel of
+// two species at reach 1 has its parameters in shared memory and spills 56 to 76 bytes.  The loads from
 // shared memory bound the kernel (76 % of the L1's wavefronts at 128^3, issue
 // slots 66 %).
 template <int S, int R, bool DRAG, int TX, int MODE>
@@ -487,8 +498,9 @@ cudaError_t launch_pass1(const mlbi_params &p, const mlbi_buffers &b, cudaStream
     if (p.tile_r == 1) return launch_pass1_tiled<S, 1, DRAG>(p, b, s);
     if (p.tile_r == 2) return launch_pass1_tiled<S, 2, DRAG>(p, b, s);
     if (p.tile_r == 3) return launch_pass1_tiled<S, 3, DRAG>(p, b, s);
-    return launch_step(k_pass1<S, DRAG, kExact>, (unsigned)((p.N + 31) / 32), dim3(32, kParts), 0, s, p, b.mom, b.dg, b.table, b.fext,
-                       b.attr, b.mom, b.frest, b.pst);
+    const auto k = p.has_attraction && !p.attr_r ? k_pass1<S, DRAG, kExact, true> : k_pass1<S, DRAG, kExact, false>;
+    return launch_step(k, (unsigned)((p.N + 31) / 32), dim3(32, kParts), 0, s, p, b.mom, b.dg, b.table, b.fext, b.attr,
+                       b.mom, b.frest, b.pst);
 }
 
 template <int S>
@@ -511,7 +523,7 @@ cudaError_t launch_sweep(const mlbi_params &p, const mlbi_buffers &b, const floa
     if (p.tile_r == 1) return launch_sweep_tiled<S, 1, DRAG>(p, b, prev, next, s);
     if (p.tile_r == 2) return launch_sweep_tiled<S, 2, DRAG>(p, b, prev, next, s);
     if (p.tile_r == 3) return launch_sweep_tiled<S, 3, DRAG>(p, b, prev, next, s);
-    return launch_step(k_pass1<S, DRAG, kSweep>, (unsigned)((p.N + 31) / 32), dim3(32, kParts), 0, s, p, prev, b.dg, b.table, b.fext,
+    return launch_step(k_pass1<S, DRAG, kSweep, false>, (unsigned)((p.N + 31) / 32), dim3(32, kParts), 0, s, p, prev, b.dg, b.table, b.fext,
                        b.attr, b.mom, b.frest, next);
 }
 

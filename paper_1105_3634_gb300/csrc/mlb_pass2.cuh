@@ -48,10 +48,11 @@ __device__ __forceinline__ void add_rest(float (&acc)[3], const float4 fr)
 }
 
 // a^a = frest^a + vx_ab sum_{+-d} s s.[(g(r)+g(r+d))/2 n^b(r+d) (u*^b(r+d) - u*^a(r))]
-// from global memory: 32 sites a block, kParts threads per site (as k_pass1)
+// from global memory: 32 sites a block, kParts threads per site (as k_pass1).  Five
+// blocks per SM, four for four species (416 bytes of spills at five, 24 at four).
 constexpr int kParts2 = 4;
 template <int S, bool DRAG>
-__global__ void __launch_bounds__(32 * kParts2, 5) k_pass2(const mlbi_params p, const float *__restrict__ dg,
+__global__ void __launch_bounds__(32 * kParts2, S == 4 && !DRAG ? 4 : 5) k_pass2(const mlbi_params p, const float *__restrict__ dg,
                                                            const mlbi_entry *__restrict__ tab,
                                                            const float4 *__restrict__ frest,
                                                            const float4 *__restrict__ pst, float4 *__restrict__ acc_f,
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(kBX * kBY, S <= 2 ? 3 : 2) k_pass2_collide(con
 // ------------------------------------------------------------------ fused, with bulk tensor copies
 // The same per-site arithmetic as k_pass2_collide.  The site's own data of a
 // plane -- its 19 S populations, moments and rest force -- arrive as three
-// bulk tensor (TMA) copies of the block's 32 x 4 sites, issued by one thread
+// bulk tensor (TMA) copies of the block's 128 sites (32 x 4 or 16 x 8), issued by one thread
 // at the top of the plane and waited on (mbarrier, bounded) only before the
 // collision, so they land while the plane's shell sums run.  Shared layouts
 // are those of the cp.async variant: population (a, i) of thread t at
