@@ -325,18 +325,16 @@ mlb_status rebuild(mlb_ctx *c)
     // gain from them.
     const bool few_warps = S == 4 && shell_reach == 2 && attr_reach > 8;
     const int tile_r = mlbi_tile_ty(S, shell_reach) && !few_warps ? shell_reach : 0;
-    auto push = [&](int dx, int dy, int dz, double vx, double vy, double vz, int mask) {
+    auto push = [&](int dx, int dy, int dz, double vx, double vy, double vz) {
         mlbi_entry e0, e1;
         e0.x = (float)vx; e0.y = (float)vy; e0.z = (float)vz;
         int packed = mlbi_pack(dx, dy, dz);
         std::memcpy(&e0.w, &packed, sizeof(int));
         long long lin = dx + nx * dy + nxy * dz;
         if (lin >= (1ll << 31) || lin <= -(1ll << 31)) lin_overflow = true;
-        int lin32 = (int)lin, zero = 0;
+        const int lin32 = (int)lin;
         std::memcpy(&e1.x, &lin32, sizeof(int));
-        std::memcpy(&e1.y, &mask, sizeof(int));
-        std::memcpy(&e1.z, &zero, sizeof(int));
-        std::memcpy(&e1.w, &zero, sizeof(int));
+        e1.y = e1.z = e1.w = 0.f;
         tab.push_back(e0);
         tab.push_back(e1);
         maxoff = std::max(maxoff, std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))));
@@ -445,7 +443,7 @@ mlb_status rebuild(mlb_ctx *c)
                             if (q == 0.0 || !canonical(dx, dy, dz)) continue;
                             if (q < sab * sab || q > rc * rc) continue;
                             const double k = 6.0 * e * s6 / (q * q * q * q);
-                            push(dx, dy, dz, k * dx, k * dy, k * dz, 0);
+                            push(dx, dy, dz, k * dx, k * dy, k * dz);
                         }
             }
             pr.attr_count = count() - pr.attr_start;

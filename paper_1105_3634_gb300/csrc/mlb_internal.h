@@ -80,7 +80,10 @@ struct mlbi_params {
 // S(S+1)/2 contact-value deviations.  Reach 3 tiles leave room for one block
 // per SM, so `split` threads share a site there (each takes every split-th
 // group of the shell table) to keep enough warps resident; their partial sums
-// meet in shared memory behind the ring.
+// meet in shared memory behind the ring.  So they do at reach 2, where the rings of three
+// and four species leave one block of 4 warps otherwise: three threads a site for three
+// species, two for the others (four: 204 KB with two).  Per step at 64^3, 1 / 1.5 / 2 and 1 / 1.5 / 1.75
+// / 2: 0.680 -> 0.279 and 1.17 -> 0.536 ms (one thread a site from global memory before).
 #define MLBI_MAX_TILE_BYTES (227 * 1024)
 struct mlbi_tile {
     int tx, ty, split;               // ty = 0: no tile, the global-memory passes
@@ -99,8 +102,8 @@ __host__ __device__ constexpr int mlbi_tile_ty(int S, int R) { return mlbi_tile_
 // Tile width of the reach-1 passes (one and two species): 32 x 4 sites, or 16
 // x 8 where that leaves at least a tenth fewer idle threads (nx = 16: half of a
 // 32-wide tile is idle; nx = 97, ny = 61: 72 % against 83 % of the threads have
-// a site).  At equal use 32 x 4 is the faster: the contact values of a warp's
-// two 16-site rows share banks.
+// a site).  At equal use the wide tiles stay: their rows are read in full lines, and in the
+// fused tiles the contact values of a narrow warp's two rows meet in 2 banks of 16.
 inline bool mlbi_narrow_tiles(int S, int tile_r, long long tiles32, long long tiles16)
 {
     return S <= 2 && tile_r == 1 && 10 * tiles16 <= 9 * tiles32;
@@ -128,6 +131,10 @@ inline long long mlbi_tile_planes(const mlbi_params &p)
 // W (1 + 1/z)/M + z + 1, least at z = sqrt(W / M).  Measured (reach 1, planes
 // per block and ms per step): 64 x 8 x 8 1: 0.020, 8: 0.056; 97 x 61 x 45 2:
 // 0.094, 12: 0.177; 128^3 6: 0.387, 12: 0.397; 256 x 16^3 4: 0.436, 12: 0.521.
+// M is the two-species bulk-copy kernels' (4 blocks per SM) for every kernel of reach 1: with the
+// fused kernels' own 2 of three and four species 64^3 took 0.120 and 0.256 ms per step against
+// 0.114 and 0.250, 128 x 128 x 96 0.564 and 1.149 against 0.569 and 1.173; with the 3 of the
+// cp.async kernel (nx % 4 != 0) nothing moved.  152: the SMs of the one part this builds for.
 constexpr int kMlbiSMs = 152;
 inline int mlbi_planes_per_block(const mlbi_params &p, long long tile_planes)
 {

@@ -21,17 +21,18 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 
 // ------------------------------------------------------------------ shared-memory tiles (z marching)
-// A block of 32 x TY threads owns a 32 x TY column of sites and marches up z
-// through `zchunk` planes.  The stencil field of every species (float4: the
+// A block owns a TX x TY column of sites (TX = 32 or 16), SPLIT threads to a site, and
+// marches up z through `zchunk` planes.  The stencil field of every species (float4: the
 // moments in pass 1, (n - n_ref, u*) in pass 2) and the contact-value
 // deviations of every pair are staged in shared memory as a ring of planes
-// of (32 + 2R) x (TY + 2R) sites: 2R + 1 planes in use and one more being
+// of (TX + 2R) x (TY + 2R) sites: 2R + 1 planes in use and one more being
 // filled by cp.async while the current plane is computed.  Every shell
 // neighbour is then read from shared memory.
-// ALT (16-wide tiles): a warp's two rows of 16 sites are two apart and the rows
-// of the contact values 24 floats, so that their 4-byte loads meet in no bank
-// (rows one apart at a pitch of 18 or 22 share most of theirs): 256 x 16^3 0.247 ->
-// 0.242 ms per step, three species at reach 3 (512 x 64 x 64) pass 2 1.061 -> 1.049.
+// ALT (16-wide tiles of pass 1, the sweeps and the split pass 2; the fused tiles do
+// without): a warp's two rows of 16 sites are two apart and the rows of the contact
+// values 24 floats, so that their 4-byte loads meet in no bank (rows one apart at a
+// pitch of 18 share 2 banks of 16, of 22 6, an extra wavefront per load): 256 x 16^3
+// 0.247 -> 0.242 ms per step, three species at reach 3 (512 x 64 x 64) pass 2 1.061 -> 1.049.
 template <int S, int R, int TY_ = kBY, int TX_ = kBX, int SPLIT_ = 1, bool ALT = false>
 struct Tile {
     static constexpr int TX = TX_, TY = TY_, SPLIT = SPLIT_;
