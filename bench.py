@@ -921,7 +921,7 @@ def run_ensemble(args, rank, world, local_rank):
                         "own_launches_value": units * steps * world / (ms_own * 1e-3) / 1e6,
                         "grouping_speedup": ms_own / ms,
                         "batch_wall_value": units * steps * world / t_batch_wall / 1e6,
-                        "autotuned_zchunks": zs,
+                        "autotuned_candidates": zs,
                         "fused_members": sum(1 for _, f in tuned if f)},
            "gpu_launches": steps * sum(sim.launches_per_step() for sim in sims),
            "clocks": clk, "e2e": None}
